@@ -175,7 +175,7 @@ __global__ void __launch_bounds__(128, MINB) k_ad_collide(const Args<S, C> a) {
   C alpha, gm[6], K[6], Vv[3];
   unpack<kABS, C>(rt, alpha, gm, K, Vv);
   C Sr[kNF];
-  bm_sources<C>(alpha, gm, K, Vv, A, D, a.slicing, Sr);
+  bm_sources<C, 3>(alpha, gm, K, Vv, A, D, a.slicing, Sr);
   C rho[kNF];
 #pragma unroll
   for (int F = 0; F < kNF; ++F) rho[F] = rt[F] + a.half_dt * Sr[F];
@@ -183,7 +183,7 @@ __global__ void __launch_bounds__(128, MINB) k_ad_collide(const Args<S, C> a) {
   {
     C alpha2, g2[6], K2[6], V2[3];
     unpack<kABS, C>(rho, alpha2, g2, K2, V2);
-    bm_flux<C, dim>(alpha2, g2, V2, A, D, Fl);
+    bm_flux<C, dim, 3>(alpha2, g2, V2, A, D, Fl);
     aQ = alpha_q<C>(a.slicing, alpha2, g2, K2);
 #pragma unroll
     for (int q = 0; q < 6; ++q) aK[q] = alpha2 * K2[q];
@@ -264,8 +264,8 @@ __global__ void __launch_bounds__(128) k_ad_init(const double* __restrict__ fiel
   double alpha, gm[6], K[6], V[3];
   unpack<kABS, double>(v, alpha, gm, K, V);
   double Sr[kNF], Fl[6][3];
-  bm_sources<double>(alpha, gm, K, V, A, D, slicing, Sr);
-  bm_flux<double, dim>(alpha, gm, V, A, D, Fl);
+  bm_sources<double, 3>(alpha, gm, K, V, A, D, slicing, Sr);
+  bm_flux<double, dim, 3>(alpha, gm, V, A, D, Fl);
   const double aQ = alpha_q<double>(slicing, alpha, gm, K);
   bool bad = false;
 #pragma unroll
@@ -323,7 +323,7 @@ __global__ void __launch_bounds__(128) k_ad_moments(const S* __restrict__ f,
   double alpha, gm[6], K[6], V[3];
   unpack<kABS, double>(rt, alpha, gm, K, V);
   double Sr[kNF];
-  bm_sources<double>(alpha, gm, K, V, A, D, slicing, Sr);
+  bm_sources<double, 3>(alpha, gm, K, V, A, D, slicing, Sr);
 #pragma unroll
   for (int F = 0; F < kNFA; ++F)
     out[(int64_t)F * G.cells + c] = F < kNF ? rt[F] + half_dt * Sr[F] : rt[F];
@@ -513,7 +513,7 @@ __global__ void __launch_bounds__(32 * (NS * P + 1), 1)
     C alpha, gm[6], K[6], Vv[3];
     unpack<kABS, C>(rt, alpha, gm, K, Vv);
     C Sr[kNF];
-    bm_sources<C>(alpha, gm, K, Vv, A, D, a.slicing, Sr);
+    bm_sources<C, 3>(alpha, gm, K, Vv, A, D, a.slicing, Sr);
     C rho[kNF];
 #pragma unroll
     for (int F = 0; F < kNF; ++F) rho[F] = rt[F] + a.half_dt * Sr[F];
@@ -521,7 +521,7 @@ __global__ void __launch_bounds__(32 * (NS * P + 1), 1)
     {
       C alpha2, g2[6], K2[6], V2[3];
       unpack<kABS, C>(rho, alpha2, g2, K2, V2);
-      bm_flux<C, dim>(alpha2, g2, V2, A, D, Fl);
+      bm_flux<C, dim, 3>(alpha2, g2, V2, A, D, Fl);
       aQ = alpha_q<C>(a.slicing, alpha2, g2, K2);
 #pragma unroll
       for (int q = 0; q < 6; ++q) aK[q] = alpha2 * K2[q];

@@ -526,7 +526,7 @@ __global__ void __launch_bounds__(128, HOLD ? 1 : MINB) k_collide(const StepArgs
   C alpha, gm[6], K[6], V[3];
   unpack<REP, C>(rt, alpha, gm, K, V);
   C Sr[kNF];
-  bm_sources<C>(alpha, gm, K, V, A, D, a.slicing, Sr);
+  bm_sources<C, dim>(alpha, gm, K, V, A, D, a.slicing, Sr);
   add_fluid(a, alpha, gm, Sr);
   C sb[3], sB[3][3];  // shift and B_k^i at this cell (SHIFT = 2)
   if (SHIFT == 1) shift_sources<C>(a.beta, alpha, A, D, Sr);
@@ -637,7 +637,7 @@ __device__ __forceinline__ void cell_terms(const StepArgs<S, C>& a, const Nbr& n
   constexpr int dim = Lattice<Q>::kDim;
   C alpha, gm[6], K[6], V[3];
   unpack<REP, C>(rt, alpha, gm, K, V);
-  bm_sources<C>(alpha, gm, K, V, A, D, a.slicing, Sr);
+  bm_sources<C, dim>(alpha, gm, K, V, A, D, a.slicing, Sr);
   add_fluid(a, alpha, gm, Sr);
   C sb[3], sB[3][3];  // shift and B_k^i at this cell (SHIFT = 2)
   if (SHIFT == 1) shift_sources<C>(a.beta, alpha, A, D, Sr);
@@ -908,7 +908,7 @@ __device__ __forceinline__ void collide_cell(const StepArgs<S, C>& a, int64_t c)
   C alpha, gm[6], K[6], V[3];
   unpack<REP, C>(rt, alpha, gm, K, V);
   C Sr[kNF];
-  bm_sources<C>(alpha, gm, K, V, A, D, a.slicing, Sr);
+  bm_sources<C, dim>(alpha, gm, K, V, A, D, a.slicing, Sr);
   add_fluid(a, alpha, gm, Sr);
   if (!a.sources_on) {
 #pragma unroll
@@ -1049,7 +1049,7 @@ __global__ void __launch_bounds__(128) k_init(const Init64Args<S> a) {
   double alpha, gm[6], K[6], V[3];
   unpack<kABS, double>(r, alpha, gm, K, V);
   double Sr[kNF];
-  bm_sources<double>(alpha, gm, K, V, A, D, a.slicing, Sr, a.fluidP);
+  bm_sources<double, Lattice<Q>::kDim>(alpha, gm, K, V, A, D, a.slicing, Sr, a.fluidP);
   double sb[3] = {a.beta[0], a.beta[1], a.beta[2]}, sB[3][3];
   if (a.beta_field) {
     shift_field_at<Q, double>(n, cells, a.beta_field, a.beta, a.inv4dx, sb, sB);
@@ -1209,7 +1209,7 @@ __global__ void __launch_bounds__(128) k_correct64(double* __restrict__ macro,
   double alpha, gm[6], K[6], V[3];
   unpack<kABS, double>(r, alpha, gm, K, V);
   double S[kNF];
-  bm_sources<double>(alpha, gm, K, V, A, D, slicing, S, fluidP);
+  bm_sources<double, Lattice<Q>::kDim>(alpha, gm, K, V, A, D, slicing, S, fluidP);
   double sb[3] = {bx, by, bz};
   if (beta_field) {
     const double b0[3] = {bx, by, bz};
