@@ -120,9 +120,10 @@ int lbnr_step(lbnr_ctx* ctx, int64_t n);
 /* Same work as lbnr_step(n), launched one kernel at a time with CUDA events
  * recorded around every launch on the context's stream; synchronises and
  * adds the elapsed milliseconds per kernel kind into ms_out[2]
- * (ms_out[0]: the moment pass feeding the derivative stencil, which LAG does
- * not run, ms_out[1]: the fused collide-and-stream kernel). For
- * measurement. */
+ * (ms_out[0]: the moment pass feeding the derivative stencil, where it is a
+ * launch of its own: not under LAG, which does not run it, nor in the forms
+ * that run both passes in one launch; ms_out[1]: the collide-and-stream kernel
+ * or that one launch). For measurement. */
 int lbnr_step_timed(lbnr_ctx* ctx, int64_t n, double* ms_out);
 
 /* Corrected macroscopic fields rho = sum_l f_l + dt S/2 (Sec. LBM), evaluated

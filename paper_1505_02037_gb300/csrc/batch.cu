@@ -113,6 +113,12 @@ __device__ bool team_sync(const BatchParams& p, const Assign& A, int k) {
   return ok != 0;
 }
 
+// Whether the collide pass takes the sums of the moment pass again: FP64 saves
+// the operations; FP32 sums every word, which brings the words on chip for the
+// second read (32 runs, FP32 deviations: 68.4 against 72.7 ms).
+template <class C>
+constexpr bool kReuse = sizeof(C) == 8;
+
 template <int Q, class S, class C, int REP, bool LAG>
 __device__ void run_steps(const BatchParams& p, const BatchRun& R, const Assign& A) {
   // every field read once into registers (a runtime index into a copy of the
@@ -124,6 +130,7 @@ __device__ void run_steps(const BatchParams& p, const BatchRun& R, const Assign&
   const int64_t start = p.done[A.run];
   StepArgs<S, C> a;
   a.aux = static_cast<const C*>(R.aux);
+  a.sums = a.aux + 7 * R.G.cells;  // SYNC: planes 7 and 8
   a.flag = &p.status[A.run];
   a.G = R.G;
   const double dx = R.dx, tau = R.tau;
@@ -161,13 +168,18 @@ __device__ void run_steps(const BatchParams& p, const BatchRun& R, const Assign&
     } else {
       for (int64_t base = A.rank * B; base < cells; base += (int64_t)A.team * B) {
         const int64_t c = base + threadIdx.x;
-        if (c < cells) aux_cell<Q, S, C, REP, kPingPong>(a.fin, aux, a.G, c);
+        if (c < cells)
+          aux_body<Q, S, C, REP, kPingPong, kCoherent>(a.fin, aux, aux + 7 * cells, cells,
+                                                       make_nbr(a.G, c), true);
       }
       if (!team_sync(p, A, k++)) return;
     }
     for (int64_t base = A.rank * B; base < cells; base += (int64_t)A.team * B) {
       const int64_t c = base + threadIdx.x;
-      if (c < cells) collide_cell<Q, S, C, REP, kPingPong, LAG>(a, c);
+      if (c < cells &&
+          collide_body<Q, S, C, REP, kPingPong, 0, false, !LAG && kReuse<C>, LAG, true, true>(
+              a, make_nbr(a.G, c), true, Plain()))
+        atomicOr(a.flag, 1);
     }
     if (!team_sync(p, A, k++)) return;
     ++s;
@@ -500,7 +512,8 @@ int lbnr_batch_create(int nruns, const lbnr_run_desc* runs, const lbnr_batch_opt
     off_f[r] = off;
     off += ((size_t)2 * 16 * qv(runs[r].vset) * ps * sb + 255) & ~(size_t)255;
     off_aux[r] = off;
-    off += (((size_t)7 * cells * cb + 255) & ~(size_t)255) * (lag ? 2 : 1);
+    off += lag ? 2 * (((size_t)7 * cells * cb + 255) & ~(size_t)255)
+               : (((size_t)9 * cells * cb + 255) & ~(size_t)255);
   }
   const size_t stage_off = off;
   off += ((size_t)16 * b->max_cells * 8 + 255) & ~(size_t)255;

@@ -100,6 +100,10 @@ struct lbnr_ctx {
   // of the next, which the collide kernel writes; under R5 only [0] is used
   // and k_aux refills it every step.
   void* aux[2] = {nullptr, nullptr};
+  // Counters of the even and the odd step's work list; each step zeroes the
+  // other's.
+  uint32_t* counters[2] = {nullptr, nullptr};
+  uint64_t counters_bytes = 0;  // of both
   LaunchCtx L;
   bool initialised = false;
   int64_t steps = 0;
@@ -176,6 +180,15 @@ int validate(const lbnr_grid* g, int vset, const lbnr_opts* o) {
   return LBNR_OK;
 }
 
+// The work list of the lattice's SYNC step. Its counters, of the even and the
+// odd step, take the front of the staging area; a lattice whose counters would
+// fill more than half of that (2.6e8 cells) runs one pass a launch.
+Schedule schedule_for(const lbnr_grid* g, int vset) {
+  Schedule s = make_schedule((uint32_t)g->nx, (uint32_t)g->ny, (uint32_t)g->nz, vset);
+  if (2 * align256(4ull * (1 + s.units)) > kStageBytes / 2) s.units = 0;
+  return s;
+}
+
 Layout layout_for(const lbnr_grid* g, int vset, int storage, int streaming, int deriv_mode) {
   const int Q = q_of(vset);
   const uint64_t cells = (uint64_t)g->nx * g->ny * g->nz;
@@ -228,6 +241,8 @@ LaunchCtx step_ctx(const lbnr_ctx* c, int64_t parity) {
     L.aux = c->aux[parity & 1];
     L.aux_out = c->aux[(parity + 1) & 1];
   }
+  L.sched.cnt = c->counters[parity & 1];
+  L.sched.cnt_next = c->counters[(parity + 1) & 1];
   return L;
 }
 
@@ -245,7 +260,7 @@ cudaError_t enqueue_step(lbnr_ctx* c, int64_t parity) {
   }
   const LaunchCtx L = step_ctx(c, parity);
   cudaError_t e = cudaSuccess;
-  if (!lagged(c)) e = c->ops->aux(L, layout, fin);
+  if (!lagged(c) && !c->ops->fused(L, c->variant)) e = c->ops->aux(L, layout, fin);
   if (e != cudaSuccess) return e;
   e = c->ops->step(L, layout, c->variant, fin, fout);
   if (e == cudaSuccess && c->L.clock) {
@@ -261,6 +276,13 @@ void drop_graphs(lbnr_ctx* c) {
       cudaGraphExecDestroy(g);
       g = nullptr;
     }
+}
+
+// A change of the step's form or parameters: the captured steps carry the old
+// ones, and the work list's counters may be left by a form that used them.
+cudaError_t form_changed(lbnr_ctx* c) {
+  drop_graphs(c);
+  return cudaMemsetAsync(c->counters[0], 0, c->counters_bytes, c->st);
 }
 
 int build_cycle(lbnr_ctx* c, int parity) {
@@ -415,7 +437,15 @@ int lbnr_create(const lbnr_grid* grid, int vset, double tau, double dx, double d
   L.partials = reinterpret_cast<double*>(b + Ly.partials);
   L.out22 = reinterpret_cast<double*>(b + Ly.out22);
   L.flag = reinterpret_cast<int*>(b + Ly.flag);
-  L.stage = b + Ly.stage;
+  // the moment pass's other two planes share the FP64 field planes, which no
+  // step keeps anything in
+  L.sums = L.macro;
+  L.sched = schedule_for(grid, vset);
+  const uint64_t counters = L.sched.units ? align256(4ull * (1 + L.sched.units)) : 0;
+  c->counters_bytes = 2 * counters;
+  c->counters[0] = reinterpret_cast<uint32_t*>(b + Ly.stage);
+  c->counters[1] = reinterpret_cast<uint32_t*>(b + Ly.stage + counters);
+  L.stage = b + Ly.stage + c->counters_bytes;
   L.st = c->st;
   L.block = 128;
   L.clock = nullptr;
@@ -439,6 +469,7 @@ int lbnr_init(lbnr_ctx* c, const double* fields) {
   const size_t nb = sizeof(double) * 16 * (size_t)c->L.cells;
   CUDA_TRY(c, cudaMemcpyAsync(c->L.macro, fields, nb, cudaMemcpyHostToDevice, c->st));
   CUDA_TRY(c, cudaMemsetAsync(c->L.flag, 0, sizeof(int), c->st));
+  CUDA_TRY(c, cudaMemsetAsync(c->counters[0], 0, c->counters_bytes, c->st));
   if (c->L.clock)
     CUDA_TRY(c, cudaMemsetAsync(const_cast<int64_t*>(c->L.clock), 0, sizeof(int64_t), c->st));
   CUDA_TRY(c, c->ops->init(c->L, c->f[0]));
@@ -503,7 +534,8 @@ int lbnr_step_timed(lbnr_ctx* c, int64_t n, double* ms_out) {
     }
     const LaunchCtx L = step_ctx(c, parity);
     cudaError_t e = cudaEventRecord(ev[0], c->st);
-    if (e == cudaSuccess && !lagged(c)) e = c->ops->aux(L, layout, fin);
+    if (e == cudaSuccess && !lagged(c) && !c->ops->fused(L, c->variant))
+      e = c->ops->aux(L, layout, fin);
     if (e == cudaSuccess) e = cudaEventRecord(ev[1], c->st);
     if (e == cudaSuccess) e = c->ops->step(L, layout, c->variant, fin, fout);
     if (e == cudaSuccess) e = cudaEventRecord(ev[2], c->st);
@@ -584,7 +616,7 @@ int lbnr_get_cells(lbnr_ctx* c, int64_t n, const int64_t* cells, double* out) {
     if (cells[i] < 0 || cells[i] >= c->L.cells)
       return fail(c, LBNR_EINVAL, "cell index %lld out of range", (long long)cells[i]);
   const int64_t per = 16 * c->Q;
-  const int64_t chunk = (int64_t)(kStageBytes / (8 * (per + 1)));
+  const int64_t chunk = (int64_t)((kStageBytes - c->counters_bytes) / (8 * (per + 1)));
   int64_t* didx = static_cast<int64_t*>(c->L.stage);
   double* dout = reinterpret_cast<double*>(didx + chunk);
   for (int64_t s = 0; s < n; s += chunk) {
@@ -609,6 +641,7 @@ int lbnr_set_distributions(lbnr_ctx* c, const double* in) {
       CUDA_TRY(c, c->ops->set_plane(c->L, layout_now(c), state_now(c), F, l, plane));
     }
   CUDA_TRY(c, cudaMemsetAsync(c->L.flag, 0, sizeof(int), c->st));
+  CUDA_TRY(c, cudaMemsetAsync(c->counters[0], 0, c->counters_bytes, c->st));
   CUDA_TRY(c, cudaStreamSynchronize(c->st));
   c->initialised = true;
   return LBNR_OK;
@@ -673,7 +706,7 @@ int lbnr_set_fluid(lbnr_ctx* c, double rho0, double w, double t0) {
   }
   c->L.fluid_P0 = w * rho0;
   c->L.fluid_t0 = t0;
-  drop_graphs(c);  // the captured steps carry the old parameters
+  CUDA_TRY(c, form_changed(c));
   return LBNR_OK;
 }
 
@@ -686,7 +719,7 @@ int lbnr_set_shift(lbnr_ctx* c, double bx, double by, double bz) {
   c->L.beta[1] = by;
   c->L.beta[2] = bz;
   c->L.shift_on = (bx != 0.0 || by != 0.0 || bz != 0.0 || c->L.beta_field) ? 1 : 0;
-  drop_graphs(c);  // the captured steps carry the old parameters
+  CUDA_TRY(c, form_changed(c));
   return LBNR_OK;
 }
 
@@ -710,7 +743,7 @@ int lbnr_set_shift_field(lbnr_ctx* c, const double* beta) {
   }
   const double* b = c->L.beta;
   c->L.shift_on = (b[0] != 0.0 || b[1] != 0.0 || b[2] != 0.0 || c->L.beta_field) ? 1 : 0;
-  drop_graphs(c);
+  CUDA_TRY(c, form_changed(c));
   return LBNR_OK;
 }
 
@@ -718,7 +751,7 @@ int lbnr_set_variant(lbnr_ctx* c, int v) {
   if (!c || v < 0 || v >= c->ops->nvariants) return fail(c, LBNR_EINVAL, "no variant %d", v);
   if (v != c->variant) {
     CUDA_TRY(c, cudaStreamSynchronize(c->st));
-    drop_graphs(c);
+    CUDA_TRY(c, form_changed(c));
     c->variant = v;
   }
   return LBNR_OK;

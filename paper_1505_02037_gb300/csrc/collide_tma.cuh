@@ -1,5 +1,5 @@
 // Bulk-copy-fed, warp-specialised form of the fused collide-and-stream step
-// (same arithmetic as k_collide_w in kernels.cuh: Eq. numlb with the
+// (same arithmetic as k_collide in kernels.cuh: Eq. numlb with the
 // equilibria and sources of Eqs. alfa-ekstsor and rho = sum f + dt S/2).
 //
 // One persistent CTA per SM. Warp NC (the producer) streams tiles of 32
@@ -215,9 +215,10 @@ __global__ void __launch_bounds__(32 * (NC + 1), 1)
     }
 
     C rho[kNF], Sr[kNF], Fl[6][3], Fv[3][3];
-    cell_terms<Q, S, C, REP>(a, n, rt, A, D, rho, Sr, Fl, Fv);
-    if (a.aux_out && valid) write_lagged<REP, C>(a.aux_out, cells, n.c, rho);
     const C three_omega = C(3) * a.omega;
+    constexpr bool kLean = lean_coefs<Q, C>;
+    cell_terms<Q, S, C, REP>(a, n, rt, A, D, kLean ? three_omega : C(1), rho, Sr, Fl, Fv);
+    if (a.aux_out && valid) write_lagged<REP, C>(a.aux_out, cells, n.c, rho);
 
 #pragma unroll
     for (int mw = 0; mw < kNF / VW; ++mw) {
@@ -225,9 +226,11 @@ __global__ void __launch_bounds__(32 * (NC + 1), 1)
 #pragma unroll
       for (int i = 0; i < VW; ++i) {
         const int F = VW * mw + i;
-        cf[i] = a.omega * rho[F] + a.sigma * Sr[F];
+        cf[i] = kLean ? a.omega * rt[F] + (a.half_dt + a.half_dt) * Sr[F]
+                      : a.omega * rho[F] + a.sigma * Sr[F];
 #pragma unroll
-        for (int k = 0; k < 3; ++k) b[i][k] = has_flux(F) ? three_omega * Fl[F - kK][k] : C(0);
+        for (int k = 0; k < 3; ++k)
+          b[i][k] = !has_flux(F) ? C(0) : kLean ? Fl[F - kK][k] : three_omega * Fl[F - kK][k];
       }
 #pragma unroll
       for (int l = 0; l < Q; ++l) {

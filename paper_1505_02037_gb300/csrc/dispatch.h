@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "schedule.h"
+
 namespace lbnr {
 
 constexpr uint64_t kStageBytes = 1ull << 20;
@@ -17,6 +19,7 @@ struct LaunchCtx {
   double dx, dt, tau;
   int slicing, sources_on;
   void* aux;        // 7 planes of the compute type (stencil input)
+  void* sums;       // SYNC: 2 more planes that the moment pass writes
   void* aux_out;    // LAG (reading R17): the step writes its corrected lapse and
                     // metric here for the next step; nullptr under R5
   double* macro;    // 16 FP64 planes (fields, moments)
@@ -37,6 +40,9 @@ struct LaunchCtx {
   double beta[3];
   int shift_on;
   const double* beta_field;
+  // The work list of the step that runs both passes in one launch, with the
+  // counters of this step (units = 0: one pass a launch).
+  Schedule sched;
 };
 
 // layout: 0 ping-pong, 1 AA at even step, 2 AA at odd step
@@ -57,6 +63,8 @@ struct Ops {
   // (aux64, plus the fields alpha and gamma into out when it is not null)
   cudaError_t (*lag_from64)(const LaunchCtx&, void* aux);
   cudaError_t (*lag_to64)(const LaunchCtx&, const void* aux, double* out);
+  // whether step() of this variant runs the moment pass itself
+  bool (*fused)(const LaunchCtx&, int variant);
 };
 
 // One getter per (velocity set, storage), each in its own translation unit

@@ -102,35 +102,61 @@ struct Impl {
     return buf[v];
   }
 
+  // Storage whose SYNC step can run both passes in one launch (k_step).
+  static constexpr bool kOneLaunch = Q == 19 && sizeof(S) == 4;
+  // Whether the step of this variant runs the moment pass itself.
+  static bool fused(const LaunchCtx& L, int variant) {
+    if (!kOneLaunch || L.sched.units == 0 || L.aux_out) return false;
+    if (L.shift_on || L.beta_field) return true;
+    const VariantSpec& x = VT::v[variant >= 0 && variant < VT::n ? variant : 0];
+    return x.kind == 0 && !x.hold;
+  }
+
+  template <int LAYOUT, int SHIFT, int TPB, int MINB>
+  static cudaError_t launch_step(const LaunchCtx& L, const StepArgs<S, C>& a) {
+    auto kern = k_step<Q, S, C, REP, LAYOUT, SHIFT, TPB, MINB>;
+    // as many blocks as fit: they claim items until none is left
+    int per_sm = 0;
+    const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, TPB, 0);
+    if (e != cudaSuccess) return e;
+    const int64_t want = ((int64_t)L.sched.items + TPB / 32 - 1) / (TPB / 32);
+    const int64_t grid = (int64_t)(per_sm > 0 ? per_sm : 1) * sm_count();
+    kern<<<(unsigned)(want < grid ? want : grid), TPB, 0, L.st>>>(a, static_cast<C*>(L.aux), static_cast<C*>(L.sums),
+                                                         L.sched);
+    return cudaGetLastError();
+  }
+
+  // One launch form: both passes in one launch (k_step), or one pass a launch.
+  // Then FP64, bound by its operations, takes the sums of the moment pass
+  // again (64^3: 867 us a step, 914 without); the other storages read every
+  // word in pass 1, which brings them on chip for pass 2 (256^3 FP16: 4.29 ms
+  // a step, 4.41 with the sums).
+  template <int LAYOUT, int SHIFT, bool H, int TPB, int MINB, int LAGMINB>
+  static cudaError_t launch_form(const LaunchCtx& L, const StepArgs<S, C>& a, bool one_launch) {
+    const unsigned grid = grid_for(L.cells, TPB);
+    if constexpr (!H && kOneLaunch) {
+      if (one_launch && !a.aux_out) return launch_step<LAYOUT, SHIFT, TPB, MINB>(L, a);
+    }
+    if (a.aux_out)
+      k_collide<Q, S, C, REP, LAYOUT, H, SHIFT, true, false, TPB, LAGMINB><<<grid, TPB, 0, L.st>>>(a);
+    else
+      k_collide<Q, S, C, REP, LAYOUT, H, SHIFT, false, sizeof(C) == 8, TPB, MINB>
+          <<<grid, TPB, 0, L.st>>>(a);
+    return cudaGetLastError();
+  }
+
   template <int LAYOUT, int VI>
-  static cudaError_t launch_generic(const LaunchCtx& L, const StepArgs<S, C>& a) {
+  static cudaError_t launch_generic(const LaunchCtx& L, const StepArgs<S, C>& a, bool one_launch) {
     constexpr VariantSpec x = VT::v[VI];
     static_assert(x.P == 1, "one thread per cell");
-    constexpr bool H = x.hold;
-    const int block = 128;
-    const int64_t threads = L.cells;
-    if constexpr (Codec<S>::kV > 1) {
-      // one thread per cell, word by word. The default shape, 128 threads
-      // sized for 3 blocks per SM with or without the lagged-field writes,
-      // takes 2 at the odd AA step, which holds a field group's Q words and
-      // reads and writes at neighbours.
-      constexpr int TPB = x.tpb > 0 ? x.tpb : 128;
-      constexpr int WMINB = x.minb > 0 ? x.minb : (LAYOUT == kAAOdd ? 2 : 3);
-      if (a.aux_out)
-        k_collide_w<Q, S, C, REP, LAYOUT, H, WMINB, true, 0, TPB>
-            <<<grid_for(threads, TPB), TPB, 0, L.st>>>(a);
-      else
-        k_collide_w<Q, S, C, REP, LAYOUT, H, WMINB, false, 0, TPB>
-            <<<grid_for(threads, TPB), TPB, 0, L.st>>>(a);
-    } else {
-      // the lagged-field writes cost registers: sized for 2 blocks per SM
-      if (a.aux_out)
-        k_collide<Q, S, C, REP, LAYOUT, H, 0, 2, true>
-            <<<grid_for(threads, block), block, 0, L.st>>>(a);
-      else
-        k_collide<Q, S, C, REP, LAYOUT, H><<<grid_for(threads, block), block, 0, L.st>>>(a);
-    }
-    return cudaGetLastError();
+    constexpr int TPB = x.tpb > 0 ? x.tpb : 128;
+    // The default shape, 128 threads sized for 3 blocks per SM, takes 2 where
+    // it would spill: word by word at the odd AA step, which holds a field
+    // group's Q words and reads and writes at neighbours, and in FP64 with the
+    // lagged-field writes.
+    constexpr int MINB = x.minb > 0 ? x.minb : (Codec<S>::kV > 1 && LAYOUT == kAAOdd ? 2 : 3);
+    constexpr int LAGMINB = Codec<S>::kV > 1 ? MINB : 2;
+    return launch_form<LAYOUT, 0, x.hold, TPB, MINB, LAGMINB>(L, a, one_launch);
   }
 
   // Registers of the shift forms. FP64 (value by value): 3 blocks of 128
@@ -140,25 +166,11 @@ struct Impl {
   // odd AA step, else 2 (255 registers; 3 would spill).
   template <int LAYOUT, int SHIFT>
   static cudaError_t launch_shifted(const LaunchCtx& L, const StepArgs<S, C>& a) {
-    constexpr int MINB = sizeof(C) == 8 ? 3 : 2;
-    constexpr int WMINB = SHIFT == 1 && LAYOUT != kAAOdd ? 3 : 2;
-    const int block = 128;
-    if constexpr (Codec<S>::kV > 1) {
-      if (a.aux_out)
-        k_collide_w<Q, S, C, REP, LAYOUT, false, WMINB, true, SHIFT>
-            <<<grid_for(L.cells, block), block, 0, L.st>>>(a);
-      else
-        k_collide_w<Q, S, C, REP, LAYOUT, false, WMINB, false, SHIFT>
-            <<<grid_for(L.cells, block), block, 0, L.st>>>(a);
-    } else {
-      if (a.aux_out)
-        k_collide<Q, S, C, REP, LAYOUT, false, SHIFT, MINB, true>
-            <<<grid_for(L.cells, block), block, 0, L.st>>>(a);
-      else
-        k_collide<Q, S, C, REP, LAYOUT, false, SHIFT, MINB>
-            <<<grid_for(L.cells, block), block, 0, L.st>>>(a);
+    if constexpr (kOneLaunch) {
+      if (fused(L, 0)) return launch_step<LAYOUT, SHIFT, 64, 4>(L, a);
     }
-    return cudaGetLastError();
+    constexpr int MINB = sizeof(C) == 8 || (SHIFT == 1 && LAYOUT != kAAOdd) ? 3 : 2;
+    return launch_form<LAYOUT, SHIFT, false, 128, MINB, MINB>(L, a, false);
   }
 
   template <int LAYOUT, int VI>
@@ -184,11 +196,11 @@ struct Impl {
   static cudaError_t launch_variant(const LaunchCtx& L, const StepArgs<S, C>& a) {
     if constexpr (VT::v[VI].kind == 1) {
       if constexpr (LAYOUT == kAAOdd)
-        return launch_generic<LAYOUT, VT::fallback>(L, a);
+        return launch_generic<LAYOUT, VT::fallback>(L, a, false);
       else
         return launch_tma<LAYOUT, VI>(L, a);
     } else {
-      return launch_generic<LAYOUT, VI>(L, a);
+      return launch_generic<LAYOUT, VI>(L, a, L.sched.units > 0);
     }
   }
 
@@ -223,6 +235,7 @@ struct Impl {
     a.fin = static_cast<const S*>(fin);
     a.fout = static_cast<S*>(fout);
     a.aux = static_cast<const C*>(L.aux);
+    a.sums = static_cast<const C*>(L.sums);
     a.aux_out = static_cast<C*>(L.aux_out);
     a.flag = L.flag;
     a.G = make_grid(L.nx, L.ny, L.nz, L.cells, L.pstride);
@@ -262,9 +275,10 @@ struct Impl {
     const unsigned grid = grid_for(L.cells, 256);
     const S* fp = static_cast<const S*>(f);
     C* ap = static_cast<C*>(L.aux);
-    if (layout == kPingPong) k_aux<Q, S, C, REP, kPingPong><<<grid, 256, 0, L.st>>>(fp, ap, G);
-    else if (layout == kAAEven) k_aux<Q, S, C, REP, kAAEven><<<grid, 256, 0, L.st>>>(fp, ap, G);
-    else k_aux<Q, S, C, REP, kAAOdd><<<grid, 256, 0, L.st>>>(fp, ap, G);
+    C* sp = static_cast<C*>(L.sums);
+    if (layout == kPingPong) k_aux<Q, S, C, REP, kPingPong><<<grid, 256, 0, L.st>>>(fp, ap, sp, G);
+    else if (layout == kAAEven) k_aux<Q, S, C, REP, kAAEven><<<grid, 256, 0, L.st>>>(fp, ap, sp, G);
+    else k_aux<Q, S, C, REP, kAAOdd><<<grid, 256, 0, L.st>>>(fp, ap, sp, G);
     return cudaGetLastError();
   }
 
@@ -367,7 +381,7 @@ struct Impl {
   static const Ops* ops() {
     static const Ops o = {VT::n,     &variant_name, &step,          &aux,       &init,
                           &sum64,    &correct64,    &constraints64, &get_plane, &set_plane,
-                          &get_cells, &lag_from64,  &lag_to64};
+                          &get_cells, &lag_from64,  &lag_to64, &fused};
     return &o;
   }
 };

@@ -3,13 +3,13 @@
 // source distributions of Eqs. alfa-ekstsor and the moment rule
 // rho = sum_l f_l + dt S / 2 (Sec. "Lattice Boltzmann Model").
 //
-// One step = k_aux (zeroth moments of alpha and gamma -> 7 planes used by the
-// derivative stencil) + the collide kernel (k_collide_w, word by word, for
-// FP32 and 16-bit storage; k_collide, value by value, for FP64; or the
-// bulk-copy-fed k_collide_tma): moments of all 16 fields, A and D by central
-// differences, sources at rho~, corrected rho, flux at rho, equilibria, BGK
-// relaxation plus source, streaming. Under LAG (reading R17) the collide
-// kernel writes the next step's stencil planes itself and k_aux goes.
+// One step = the moment pass (zeroth moments of alpha and gamma -> planes used
+// by the derivative stencil) + the collide pass: moments of all 16 fields, A
+// and D by central differences, sources at rho~, corrected rho, flux at rho,
+// equilibria, BGK relaxation plus source, streaming. k_step runs both in one
+// launch; else k_aux and then k_collide (one thread per cell) or the
+// bulk-copy-fed k_collide_tma. Under LAG (reading R17) the collide kernel
+// writes the next step's stencil planes itself and there is no moment pass.
 //
 // Memory: tile-blocked words (fidx below). The 16 Q values of 32 consecutive
 // cells (x fastest) form one block; a word holds kV fields of one cell and
@@ -39,6 +39,7 @@
 
 #include "lattice.cuh"
 #include "physics.cuh"
+#include "schedule.h"
 
 namespace lbnr {
 
@@ -209,26 +210,6 @@ __host__ __device__ constexpr bool is_v(int F) { return F >= kV && F < kNF; }
 // ---------------------------------------------------------------------------
 // Geometry of one cell and its neighbours (periodic)
 // ---------------------------------------------------------------------------
-// n / d for n < 2^31 by a multiply-high with a precomputed round-up
-// multiplier (Granlund-Montgomery); d = 1 is passed through.
-struct FastDiv {
-  uint32_t d, mul, shift;
-  __device__ __forceinline__ uint32_t div(uint32_t n) const {
-    return d == 1 ? n : (__umulhi(n, mul) >> shift);
-  }
-};
-inline FastDiv make_fastdiv(uint32_t d) {
-  FastDiv f{d, 0, 0};
-  if (d > 1) {
-    uint32_t l = 0;
-    while ((1ull << l) < d) ++l;  // ceil(log2 d)
-    const uint32_t p = 31 + l;
-    f.mul = (uint32_t)(((1ull << p) + d - 1) / d);
-    f.shift = p - 32;
-  }
-  return f;
-}
-
 struct Grid {
   int32_t nx, ny, nz;
   int64_t cells;    // < 2^31 (32-bit cell indices)
@@ -333,6 +314,7 @@ struct StepArgs {
   const S* fin;
   S* fout;
   const C* aux;  // 7 planes: ln(alpha~) or log1p(alpha~ - 1); gamma~ or gamma~ - delta
+  const C* sums; // SYNC: 2 planes the moment pass writes beside them (aux_body)
   // Reading R17 (LAG): aux holds the previous step's corrected lapse and
   // metric in that form, and the step writes its own corrected ones to
   // aux_out for the next step. nullptr: aux holds this step's rho~ (R5).
@@ -428,21 +410,23 @@ __device__ __forceinline__ void shift_field_at(const Nbr& n, int64_t cells,
 }
 
 // A_k and D_kij by central differences of the aux planes (reading: second
-// order differences of ln alpha and gamma_ij / 2).
-template <int Q, class C>
+// order differences of ln alpha and gamma_ij / 2). COH: the planes are written
+// by the same launch, so the loads bypass L1.
+template <int Q, class C, bool COH = false>
 __device__ __forceinline__ void derivatives(const Nbr& n, int64_t cells, const C* __restrict__ aux,
                                             C inv2dx, C inv4dx, C A[3], C D[3][6]) {
   constexpr int dim = Lattice<Q>::kDim;
+  auto ld = [](const C* p) { return COH ? __ldcg(p) : __ldg(p); };
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
     if (k < dim) {
       const uint32_t cp = n.at(k == 0, k == 1, k == 2);
       const uint32_t cm = n.at(-(k == 0), -(k == 1), -(k == 2));
-      A[k] = (__ldg(aux + cp) - __ldg(aux + cm)) * inv2dx;
+      A[k] = (ld(aux + cp) - ld(aux + cm)) * inv2dx;
 #pragma unroll
       for (int q = 0; q < 6; ++q) {
         const C* plane = aux + (size_t)(1 + q) * (size_t)cells;
-        D[k][q] = (__ldg(plane + cp) - __ldg(plane + cm)) * inv4dx;
+        D[k][q] = (ld(plane + cp) - ld(plane + cm)) * inv4dx;
       }
     } else {
       A[k] = C(0);
@@ -466,174 +450,15 @@ __device__ __forceinline__ void unpack(const C m[kNF], C& alpha, C g[6], C K[6],
   for (int k = 0; k < 3; ++k) V[k] = m[kV + k];
 }
 
-// ---------------------------------------------------------------------------
-// k_collide: the fused step, one thread per cell, value by value (FP64)
-// ---------------------------------------------------------------------------
-// Storage with one value per distribution word: FP64 (FP32 and 16-bit
-// storage take k_collide_w below). SHIFT: the shift terms are compiled in: 1
-// a constant shift (a.beta), 2 a static field on top of it (a.beta_field,
-// with its B terms). The zero-shift forms (0) keep none of their code or
-// registers. MINB: blocks per SM the registers are sized for (without HOLD).
-// LAGW: the form writes the lagged fields of reading R17 to a.aux_out
-// (compiled in only where asked, so the other forms keep their registers).
-template <int Q, class S, class C, int REP, int LAYOUT, bool HOLD, int SHIFT = 0, int MINB = 3,
-          bool LAGW = false>
-__global__ void __launch_bounds__(128, HOLD ? 1 : MINB) k_collide(const StepArgs<S, C> a) {
-  using L = Lattice<Q>;
-  constexpr int dim = L::kDim;
-  const int64_t cell = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const bool valid = cell < a.G.cells;
-  const int64_t c = valid ? cell : a.G.cells - 1;
-  const int64_t cells = a.G.cells;
-  const Nbr n = make_nbr(a.G, c);
-
-  // source and destination cell of each velocity
-  uint32_t rc[Q], wc[Q];
-#pragma unroll
-  for (int l = 0; l < Q; ++l) {
-    rc[l] = read_cell<Q, LAYOUT>(n, l);
-    wc[l] = write_cell<Q, LAYOUT>(n, l);
-  }
-
-  // Pass 1: zeroth moments (ascending l).
-  C fv[HOLD ? kNF : 1][HOLD ? Q : 1];
-  C rt[kNF];
-#pragma unroll
-  for (int F = 0; F < kNF; ++F) {
-    C s = C(0);
-#pragma unroll
-    for (int l = 0; l < Q; ++l) {
-      // In place (AA) the buffer is written by this kernel: re-read values
-      // must come through coherent loads, never the read-only path.
-      const S* src = a.fin + fidx<Q, S>(rc[l], F, read_slot<LAYOUT>(l));
-      const C v = HOLD ? Codec<S>::load(src)
-                  : LAYOUT == kPingPong ? Codec<S>::load_keep(src) : Codec<S>::load_coh(src);
-      if (HOLD) fv[HOLD ? F : 0][HOLD ? l : 0] = v;
-      s += REP == kDEV ? C(L::w(l)) * v : v;
-    }
-    rt[F] = s;
-  }
-  {
-    C chk = C(0);
-#pragma unroll
-    for (int F = 0; F < kNF; ++F) chk += rt[F];
-    if (valid && !isfinite(chk)) atomicOr(a.flag, 1);
-  }
-
-  // Derivatives, sources at rho~, corrected rho, flux at rho.
-  C A[3], D[3][6];
-  derivatives<Q, C>(n, cells, a.aux, a.inv2dx, a.inv4dx, A, D);
-  C alpha, gm[6], K[6], V[3];
-  unpack<REP, C>(rt, alpha, gm, K, V);
-  C Sr[kNF];
-  bm_sources<C, dim>(alpha, gm, K, V, A, D, a.slicing, Sr);
-  add_fluid(a, alpha, gm, Sr);
-  C sb[3], sB[3][3];  // shift and B_k^i at this cell (SHIFT = 2)
-  if (SHIFT == 1) shift_sources<C>(a.beta, alpha, A, D, Sr);
-  if (SHIFT == 2) {
-    shift_field_at<Q, C>(n, cells, a.beta_field, a.beta, (double)a.inv4dx, sb, sB);
-    shift_sources<C>(sb, alpha, A, D, Sr);
-    shift_field_sources<C>(gm, K, V, D, sB, Sr);
-  }
-  if (!a.sources_on) {
-#pragma unroll
-    for (int F = 0; F < kNF; ++F) Sr[F] = C(0);
-  }
-  C rho[kNF];  // ABS: rho; DEV: rho - rho_flat
-#pragma unroll
-  for (int F = 0; F < kNF; ++F) rho[F] = rt[F] + a.half_dt * Sr[F];
-  if (LAGW && valid) write_lagged<REP, C>(a.aux_out, cells, n.c, rho);
-  C Fl[6][3];
-  C Fv[SHIFT == 2 ? 3 : 1][3];  // V fluxes under a shift field
-  {
-    C alpha2, g2[6], K2[6], V2[3];
-    unpack<REP, C>(rho, alpha2, g2, K2, V2);
-    bm_flux<C, dim>(alpha2, g2, V2, A, D, Fl);
-    if (SHIFT == 1) shift_flux_k<C, dim>(a.beta, K2, Fl);
-    if (SHIFT == 2) {
-      shift_flux_k<C, dim>(sb, K2, Fl);
-      shift_field_vflux<C, dim>(g2, V2, sb, sB, Fv);
-    }
-  }
-  // Per-field coefficients: coef = omega rho + sigma S; flux scaled by 3 omega.
-  C coef[kNF];
-#pragma unroll
-  for (int F = 0; F < kNF; ++F) coef[F] = a.omega * rho[F] + a.sigma * Sr[F];
-  const C three_omega = C(3) * a.omega;
-
-  // Pass 2: relax, add the source, stream.
-#pragma unroll
-  for (int F = 0; F < kNF; ++F) {
-    const C cf = coef[F];
-    C b[3] = {C(0), C(0), C(0)};
-    if (has_flux(F)) {
-#pragma unroll
-      for (int k = 0; k < dim; ++k) b[k] = three_omega * Fl[F - kK][k];
-    }
-    // under a shift the V fields take the flux -beta^k V_i
-    const bool vflux = SHIFT && is_v(F);
-    // All Q values of this field are read before any is written: in place
-    // (AA) the field's reads and writes touch the same Q locations.
-    C v_[Q];
-#pragma unroll
-    for (int l = 0; l < Q; ++l) {
-      const S* src = a.fin + fidx<Q, S>(rc[l], F, read_slot<LAYOUT>(l));
-      // the second read is the last use: streaming (evict-first) load
-      v_[l] = HOLD ? fv[HOLD ? F : 0][HOLD ? l : 0]
-              : LAYOUT == kPingPong ? Codec<S>::load(src) : Codec<S>::load_coh(src);
-    }
-    if (vflux && SHIFT == 2) {
-#pragma unroll
-      for (int k = 0; k < dim; ++k) b[k] = three_omega * Fv[SHIFT == 2 ? F - kV : 0][k];
-    } else if (vflux) {
-      // V_i at the corrected moments, recovered from this field's own values
-      // rather than kept live since pass 1: coef = omega rho~ + dt S (as
-      // omega dt/2 + sigma = dt), so rho = rho~ + (coef - omega rho~) / 2.
-      C s = C(0);
-#pragma unroll
-      for (int l = 0; l < Q; ++l) s += REP == kDEV ? C(L::w(l)) * v_[l] : v_[l];
-      const C mv = -three_omega * (s + C(0.5) * (cf - a.omega * s));
-#pragma unroll
-      for (int k = 0; k < dim; ++k) b[k] = mv * a.beta[k];
-    }
-    // FP64 (bound by its arithmetic): w_l (cf + c.b) as w_l cf + c.(w_l b),
-    // whose products repeat across velocities of equal weight and are formed
-    // once each, instead of one product per velocity
-    constexpr bool kLeanRelax = sizeof(C) == 8 && REP == kABS;
-#pragma unroll
-    for (int l = 0; l < Q; ++l) {
-      const C v = v_[l];
-      C t = kLeanRelax ? C(L::w(l)) * cf : cf;
-      if (has_flux(F) || vflux) {
-#pragma unroll
-        for (int k = 0; k < dim; ++k) {
-          const C bk = kLeanRelax ? C(L::w(l)) * b[k] : b[k];
-          if (L::c(l, k) > 0) t += bk;
-          if (L::c(l, k) < 0) t -= bk;
-        }
-      }
-      const C out = REP == kDEV ? fma(a.omc, v, t)
-                                : (kLeanRelax ? fma(a.omc, v, t) : fma(a.omc, v, C(L::w(l)) * t));
-      // Ping-pong: lanes past the last cell were clamped to it and write the
-      // same bytes as its own lanes, so every store can be unconditional.
-      S* dst = a.fout + fidx<Q, S>(wc[l], F, write_slot<LAYOUT>(l));
-      if (LAYOUT == kPingPong)
-        Codec<S>::store(dst, out);
-      else
-        Codec<S>::store_if(dst, out, valid);
-    }
-  }
-}
-
 // From one cell's zeroth moments rt and stencil derivatives A, D: the
 // sources S at rt, the corrected moments rho = rt + dt/2 S (the moment rule
 // of the forced scheme) and the fluxes at rho. SHIFT = 1 adds the terms of a
 // constant shift a.beta, SHIFT = 2 those of the static shift field (with its
-// B_k^i) and the V fluxes -beta^k V_i it gives (Fv).
+// B_k^i) and the V fluxes -beta^k V_i it gives (Fv). `fs` scales every flux.
 template <int Q, class S, class C, int REP, int SHIFT = 0>
 __device__ __forceinline__ void cell_terms(const StepArgs<S, C>& a, const Nbr& n, const C rt[kNF],
-                                           const C A[3], const C D[3][6], C rho[kNF], C Sr[kNF],
-                                           C Fl[6][3], C Fv[3][3]) {
+                                           const C A[3], const C D[3][6], C fs, C rho[kNF],
+                                           C Sr[kNF], C Fl[6][3], C Fv[3][3]) {
   constexpr int dim = Lattice<Q>::kDim;
   C alpha, gm[6], K[6], V[3];
   unpack<REP, C>(rt, alpha, gm, K, V);
@@ -654,64 +479,211 @@ __device__ __forceinline__ void cell_terms(const StepArgs<S, C>& a, const Nbr& n
   for (int F = 0; F < kNF; ++F) rho[F] = rt[F] + a.half_dt * Sr[F];
   C alpha2, g2[6], K2[6], V2[3];
   unpack<REP, C>(rho, alpha2, g2, K2, V2);
-  bm_flux<C, dim>(alpha2, g2, V2, A, D, Fl);
-  if (SHIFT == 1) shift_flux_k<C, dim>(a.beta, K2, Fl);
+  bm_flux<C, dim>(alpha2 * fs, g2, V2, A, D, Fl);
+  if (SHIFT == 1) {
+    const C bs[3] = {fs * a.beta[0], fs * a.beta[1], fs * a.beta[2]};
+    shift_flux_k<C, dim>(bs, K2, Fl);
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+      for (int k = 0; k < 3; ++k) Fv[i][k] = -bs[k] * V2[i];
+  }
   if (SHIFT == 2) {
-    shift_flux_k<C, dim>(sb, K2, Fl);
+    const C bs[3] = {fs * sb[0], fs * sb[1], fs * sb[2]};
+    shift_flux_k<C, dim>(bs, K2, Fl);
     shift_field_vflux<C, dim>(g2, V2, sb, sB, Fv);
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+      for (int k = 0; k < 3; ++k) Fv[i][k] *= fs;
   }
 }
 
-// ---------------------------------------------------------------------------
-// k_collide_w: one thread per cell for FP32 and 16-bit storage, word by word
-// ---------------------------------------------------------------------------
-// The step of k_collide with every load and store moving a whole word of kV
-// consecutive fields of one (cell, velocity): a kV-th of the memory
-// instructions of value-by-value access. HOLD keeps the words of a
-// cell in registers between the passes. SHIFT as in k_collide: 1 a constant
-// shift, 2 a static shift field; under a shift the V fields take the flux
-// -beta^k V_i at the corrected moments. TPB: threads per block.
-template <int Q, class S, class C, int REP, int LAYOUT, bool HOLD, int MINB = 3, bool LAGW = false,
-          int SHIFT = 0, int TPB = 128>
-__global__ void __launch_bounds__(TPB, HOLD ? 1 : MINB) k_collide_w(const StepArgs<S, C> a) {
-  using L = Lattice<Q>;
-  using IO = WordIO<S>;
-  using W = typename IO::W;
-  constexpr int V = Codec<S>::kV;
-  static_assert(V > 1 && kNF % V == 0, "word access: several fields per word");
-  constexpr int NW = kNF / V;
-  const int64_t cell = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const bool valid = cell < a.G.cells;
-  const int64_t c = valid ? cell : a.G.cells - 1;
-  const int64_t cells = a.G.cells;
-  const Nbr n = make_nbr(a.G, c);
+// Fluxes carry their factor 3 omega (and in FP64 a weight) from the start, and
+// the relaxation coefficient is omega rho~ + dt S, except in the FP32 forms that
+// keep their arithmetic (bm_sources_plain) and run value by value.
+template <int Q, class C>
+constexpr bool lean_coefs = sizeof(C) == 8 || Lattice<Q>::kDim == 3;
 
-  // Pass 1: zeroth moments, kV fields per load (ascending l).
-  W hw[HOLD ? NW : 1][HOLD ? Q : 1];
-  C rt[kNF];
+// ---------------------------------------------------------------------------
+// Word access and packed FP32 arithmetic of the step
+// ---------------------------------------------------------------------------
+// How a distribution word is loaded: through the read-only path (kept for the
+// update pass), streamed (its last use), or coherently through L2 (buffers
+// that the same launch writes).
+enum : int { kKeep = 0, kLast = 1, kCoherent = 2 };
+template <class S, int POL>
+__device__ __forceinline__ typename Codec<S>::W load_word(const S* p) {
+  if constexpr (Codec<S>::kV == 1)
+    return POL == kKeep ? Codec<S>::load_keep(p) : POL == kLast ? Codec<S>::load(p) : Codec<S>::load_coh(p);
+  else
+    return POL == kKeep ? WordIO<S>::ldw_keep(p) : POL == kLast ? WordIO<S>::ldw(p) : WordIO<S>::ldw_coh(p);
+}
+// The four FP32 values of a word as two pairs. Sums, relaxation and fluxes run
+// on pairs (one instruction for two values, each rounded as by the scalar
+// instruction): 16-bit storage is bound by issue slots, and the other forms
+// wait less between their loads.
+__device__ __forceinline__ float2 pair(float a) { return make_float2(a, a); }
+__device__ __forceinline__ float2 neg(float2 a) { return make_float2(-a.x, -a.y); }
+template <class S>
+__device__ __forceinline__ void unpack_pairs(typename Codec<S>::W w, float2 v[2]) {
+  float t[4];
+  Codec<S>::unpack(w, t);
+  v[0] = make_float2(t[0], t[1]);
+  v[1] = make_float2(t[2], t[3]);
+}
+
+// Zeroth moments of the kV fields of a word at a cell (ascending l); word(l)
+// loads it.
+template <int Q, class S, class C, int REP, class Word>
+__device__ __forceinline__ void sum_words(Word word, C* sum) {
+  using L = Lattice<Q>;
+  constexpr int V = Codec<S>::kV;
+  if constexpr (V == 1) {
+    C s = C(0);
 #pragma unroll
-  for (int m = 0; m < NW; ++m) {
-    C sum[V];
+    for (int l = 0; l < Q; ++l) {
+      const C v = word(l);
+      s += REP == kDEV ? C(L::w(l)) * v : v;
+    }
+    sum[0] = s;
+  } else if constexpr (!lean_coefs<Q, C>) {
 #pragma unroll
     for (int i = 0; i < V; ++i) sum[i] = C(0);
 #pragma unroll
     for (int l = 0; l < Q; ++l) {
-      // in place (AA) the buffer is written by this kernel: coherent loads
-      const S* src = a.fin + read_index<Q, LAYOUT, S>(n, V * m, l);
-      const W w = HOLD ? IO::ldw(src) : LAYOUT == kPingPong ? IO::ldw_keep(src) : IO::ldw_coh(src);
-      if (HOLD) hw[HOLD ? m : 0][HOLD ? l : 0] = w;
       C v[V];
-      Codec<S>::unpack(w, v);
+      Codec<S>::unpack(word(l), v);
 #pragma unroll
       for (int i = 0; i < V; ++i) sum[i] += REP == kDEV ? C(L::w(l)) * v[i] : v[i];
     }
+  } else {
+    float2 s[2] = {pair(0.f), pair(0.f)};
 #pragma unroll
-    for (int i = 0; i < V; ++i) rt[V * m + i] = sum[i];
+    for (int l = 0; l < Q; ++l) {
+      float2 v[2];
+      unpack_pairs<S>(word(l), v);
+#pragma unroll
+      for (int p = 0; p < 2; ++p)
+        s[p] = REP == kDEV ? __ffma2_rn(pair((float)L::w(l)), v[p], s[p]) : __fadd2_rn(s[p], v[p]);
+    }
+    sum[0] = s[0].x;
+    sum[1] = s[0].y;
+    sum[2] = s[1].x;
+    sum[3] = s[1].y;
   }
-  // Non-finite moments are reported, and the lagged fields written, only
-  // after the update pass: a global write here (the flag or aux_out may
-  // alias the input as far as the compiler knows) would keep the update
-  // pass's loads from being issued ahead of the physics.
+}
+template <int Q, class S, class C, int REP, int LAYOUT, int POL>
+__device__ __forceinline__ void word_sums(const S* __restrict__ f, const Nbr& n, int m, C* sum) {
+  sum_words<Q, S, C, REP>(
+      [&](int l) { return load_word<S, POL>(f + read_index<Q, LAYOUT, S>(n, Codec<S>::kV * m, l)); },
+      sum);
+}
+
+// ---------------------------------------------------------------------------
+// The moment pass of one cell: stencil planes and the sums the step reuses
+// ---------------------------------------------------------------------------
+// aux: ln(alpha~) and gamma~ (or their deviations) for the stencil; sums:
+// alpha~ itself and (words of four fields) the other field of the second word,
+// K_xx. With them the collide pass needs no sums of the words that this pass
+// has summed already.
+template <class S>
+constexpr int kAuxWords = Codec<S>::kV == 1 ? 7 : 2;  // words holding fields 0..6
+template <int Q, class S, class C, int REP, int LAYOUT, int POL>
+__device__ __forceinline__ void aux_body(const S* __restrict__ f, C* __restrict__ aux, C* sums,
+                                         int64_t cells, const Nbr& n, bool valid) {
+  constexpr int V = Codec<S>::kV;
+  C s[kAuxWords<S> * V];
+#pragma unroll
+  for (int m = 0; m < kAuxWords<S>; ++m) word_sums<Q, S, C, REP, LAYOUT, POL>(f, n, m, s + V * m);
+  if (!valid) return;
+  sums[n.c] = s[0];
+  if (V > 1) sums[cells + n.c] = s[V > 1 ? 7 : 0];
+  C* p = aux + n.c;
+  p[0] = REP == kDEV ? log1p(s[0]) : log(s[0]);
+#pragma unroll
+  for (int F = 1; F < 7; ++F) p[F * cells] = s[F];
+}
+
+// ---------------------------------------------------------------------------
+// The fused step of one cell
+// ---------------------------------------------------------------------------
+// Pass 1 sums the moments, pass 2 reads the values again (from cache where
+// they survive; HOLD keeps them in registers instead), relaxes, adds the
+// source and streams, whole words of kV fields at a time. SUMS: the moments of
+// the words that the moment pass has summed come from its planes, and pass 1
+// reads only the others. SHIFT: the shift terms are compiled in: 1 a constant
+// shift (a.beta), 2 a static field on top of it (a.beta_field, with its B
+// terms); the zero-shift forms (0) keep none of their code or registers. LAGW:
+// the lagged fields of reading R17 are written to a.aux_out. COHF, COHA: the
+// distributions, the planes are written by the same launch, so their loads are
+// coherent (L1 bypassed). valid: the cell is not a clamped one past the end.
+// Hooks: what a caller adds (see Plain).
+// Returns whether a moment was not finite. The caller reports it after the
+// update pass: a global write between the passes (the flag or aux_out may
+// alias the input as far as the compiler knows) would keep pass 2's loads from
+// being issued ahead of the physics.
+struct Plain {
+  __device__ void before_planes() {}  // runs before the planes are read
+};
+template <class Before>
+struct Hooked {
+  Before before;
+  __device__ __forceinline__ void before_planes() { before(); }
+};
+template <int Q, class S, class C, int REP, int LAYOUT, int SHIFT, bool HOLD, bool SUMS, bool LAGW,
+          bool COHF, bool COHA, class Hooks>
+__device__ __forceinline__ bool collide_body(const StepArgs<S, C>& a, const Nbr& n, bool valid,
+                                             Hooks hooks) {
+  using L = Lattice<Q>;
+  using W = typename Codec<S>::W;
+  constexpr int V = Codec<S>::kV;
+  constexpr int NW = kNF / V;
+  constexpr int dim = L::kDim;
+  // in place (AA) the buffer is written by this kernel: coherent loads
+  constexpr bool kCoh = COHF || LAYOUT != kPingPong;
+  constexpr int POL1 = kCoh ? kCoherent : HOLD ? kLast : kKeep;
+  constexpr int POL2 = kCoh ? kCoherent : kLast;
+  constexpr bool kLean = lean_coefs<Q, C>;
+  constexpr bool kWeighted = sizeof(C) == 8 && REP == kABS;
+  constexpr double kWb = L::w(Q - 1);  // the weight that FP64 fluxes carry
+  const int64_t cells = a.G.cells;
+
+  W hw[HOLD ? NW : 1][HOLD ? Q : 1];
+  C rt[kNF];
+  if constexpr (HOLD) {
+#pragma unroll
+    for (int m = 0; m < NW; ++m) {
+#pragma unroll
+      for (int l = 0; l < Q; ++l)
+        hw[m][l] = load_word<S, POL1>(a.fin + read_index<Q, LAYOUT, S>(n, V * m, l));
+      C sum[V];
+#pragma unroll
+      for (int i = 0; i < V; ++i) sum[i] = C(0);
+#pragma unroll
+      for (int l = 0; l < Q; ++l) {
+        C v[V];
+        unpack_word<S>(hw[m][l], v);
+#pragma unroll
+        for (int i = 0; i < V; ++i) sum[i] += REP == kDEV ? C(L::w(l)) * v[i] : v[i];
+      }
+#pragma unroll
+      for (int i = 0; i < V; ++i) rt[V * m + i] = sum[i];
+    }
+  } else {
+#pragma unroll
+    for (int m = SUMS ? kAuxWords<S> : 0; m < NW; ++m)
+      word_sums<Q, S, C, REP, LAYOUT, POL1>(a.fin, n, m, rt + V * m);
+  }
+  hooks.before_planes();
+  if constexpr (SUMS && !HOLD) {
+    const C* p = a.aux + n.c;
+    const C* q = a.sums + n.c;
+    rt[0] = COHA ? __ldcg(q) : __ldg(q);
+#pragma unroll
+    for (int F = 1; F < 7; ++F) rt[F] = COHA ? __ldcg(p + F * cells) : __ldg(p + F * cells);
+    if (V > 1) rt[7] = COHA ? __ldcg(q + cells) : __ldg(q + cells);
+  }
   bool bad;
   {
     C chk = C(0);
@@ -721,268 +693,76 @@ __global__ void __launch_bounds__(TPB, HOLD ? 1 : MINB) k_collide_w(const StepAr
   }
 
   C A[3], D[3][6];
-  derivatives<Q, C>(n, cells, a.aux, a.inv2dx, a.inv4dx, A, D);
-  C rho[kNF], Sr[kNF], Fl[6][3], Fv[3][3];
-  cell_terms<Q, S, C, REP, SHIFT>(a, n, rt, A, D, rho, Sr, Fl, Fv);
+  derivatives<Q, C, COHA>(n, cells, a.aux, a.inv2dx, a.inv4dx, A, D);
   const C three_omega = C(3) * a.omega;
+  C rho[kNF], Sr[kNF], Fl[6][3], Fv[3][3];
+  cell_terms<Q, S, C, REP, SHIFT>(a, n, rt, A, D,
+                                  !kLean ? C(1) : kWeighted ? three_omega * C(kWb) : three_omega,
+                                  rho, Sr, Fl, Fv);
+  // cf = omega rho + sigma S = omega rho~ + dt S
+  C cf[kNF];
+#pragma unroll
+  for (int F = 0; F < kNF; ++F)
+    cf[F] = kLean ? a.omega * rt[F] + (a.half_dt + a.half_dt) * Sr[F]
+                  : a.omega * rho[F] + a.sigma * Sr[F];
+  auto flux = [&](int F, int k) -> C {
+    if (has_flux(F)) return kLean ? Fl[F - kK][k] : three_omega * Fl[F - kK][k];
+    if (SHIFT && is_v(F)) {
+      if (!kLean && SHIFT == 1) return -three_omega * rho[F] * a.beta[k];
+      return kLean ? Fv[F - kV][k] : three_omega * Fv[F - kV][k];
+    }
+    return C(0);
+  };
+  auto fluxed = [](int F) constexpr { return has_flux(F) || (SHIFT && is_v(F)); };
 
-  // Pass 2: relax, add the source, stream; all Q words of a field group are
-  // read before any is written (in place they share the Q locations).
+  // Pass 2: all Q words of a field group are read before any is written (in
+  // place they share the Q locations).
 #pragma unroll
   for (int m = 0; m < NW; ++m) {
     W vw[Q];
 #pragma unroll
-    for (int l = 0; l < Q; ++l) {
-      const S* src = a.fin + read_index<Q, LAYOUT, S>(n, V * m, l);
+    for (int l = 0; l < Q; ++l)
       vw[l] = HOLD ? hw[HOLD ? m : 0][HOLD ? l : 0]
-              : LAYOUT == kPingPong ? IO::ldw(src) : IO::ldw_coh(src);
-    }
-    C cf[V], b[V][3];
+                   : load_word<S, POL2>(a.fin + read_index<Q, LAYOUT, S>(n, V * m, l));
+    if constexpr (V == 1) {
+      C b[3];
 #pragma unroll
-    for (int i = 0; i < V; ++i) {
-      const int F = V * m + i;
-      cf[i] = a.omega * rho[F] + a.sigma * Sr[F];
-#pragma unroll
-      for (int k = 0; k < 3; ++k) {
-        C bk = has_flux(F) ? three_omega * Fl[F - kK][k] : C(0);
-        if (SHIFT == 1 && is_v(F)) bk = -three_omega * rho[F] * a.beta[k];
-        if (SHIFT == 2 && is_v(F)) bk = three_omega * Fv[SHIFT == 2 && is_v(F) ? F - kV : 0][k];
-        b[i][k] = bk;
-      }
-    }
-#pragma unroll
-    for (int l = 0; l < Q; ++l) {
-      C v[V], out[V];
-      Codec<S>::unpack(vw[l], v);
-#pragma unroll
-      for (int i = 0; i < V; ++i) {
-        C t = cf[i];
-        if (has_flux(V * m + i) || (SHIFT && is_v(V * m + i))) {
-#pragma unroll
-          for (int k = 0; k < L::kDim; ++k) {
-            if (L::c(l, k) > 0) t += b[i][k];
-            if (L::c(l, k) < 0) t -= b[i][k];
-          }
-        }
-        out[i] = REP == kDEV ? fma(a.omc, v[i], t) : fma(a.omc, v[i], C(L::w(l)) * t);
-      }
-      S* dst = a.fout + write_index<Q, LAYOUT, S>(n, V * m, l);
-      if (LAYOUT == kPingPong)
-        IO::stw(dst, Codec<S>::pack(out));
-      else
-        IO::stw_if(dst, Codec<S>::pack(out), valid);
-    }
-  }
-  if (LAGW && valid) write_lagged<REP, C>(a.aux_out, cells, n.c, rho);
-  if (bad) atomicOr(a.flag, 1);
-}
-
-// ---------------------------------------------------------------------------
-// k_aux: ln(alpha~) and gamma~ (or their deviations) for the stencil
-// ---------------------------------------------------------------------------
-template <int Q, class S, class C, int REP, int LAYOUT>
-__global__ void __launch_bounds__(256) k_aux(const S* __restrict__ f, C* __restrict__ aux, Grid G) {
-  using L = Lattice<Q>;
-  const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= G.cells) return;
-  constexpr int V = Codec<S>::kV;
-  constexpr int NW = (7 + V - 1) / V;  // the words holding fields 0..6
-  const Nbr n = make_nbr(G, c);
-  C s[NW * V];
-#pragma unroll
-  for (int F = 0; F < NW * V; ++F) s[F] = C(0);
-#pragma unroll
-  for (int m = 0; m < NW; ++m) {
-#pragma unroll
-    for (int l = 0; l < Q; ++l) {
-      const S* src = f + read_index<Q, LAYOUT, S>(n, V * m, l);
-      C v[V];
-      if constexpr (V > 1)
-        Codec<S>::unpack(WordIO<S>::ldw_keep(src), v);
-      else
-        v[0] = Codec<S>::load_keep(src);
-#pragma unroll
-      for (int i = 0; i < V; ++i)
-        if (V * m + i < 7) s[V * m + i] += REP == kDEV ? C(L::w(l)) * v[i] : v[i];
-    }
-  }
-  s[0] = REP == kDEV ? log1p(s[0]) : log(s[0]);
-#pragma unroll
-  for (int F = 0; F < 7; ++F) aux[(int64_t)F * G.cells + c] = s[F];
-}
-
-// ---------------------------------------------------------------------------
-// Per-cell bodies for kernels that run many steps in one launch (the batched
-// ensemble). Other thread blocks of the same launch write the buffers these
-// read, so every load is coherent (L1 bypassed). Same arithmetic, in the
-// same order, as k_aux and k_collide with one thread per cell.
-// ---------------------------------------------------------------------------
-template <int Q, class S, class C, int REP, int LAYOUT>
-__device__ __forceinline__ void aux_cell(const S* __restrict__ f, C* __restrict__ aux,
-                                         const Grid& G, int64_t c) {
-  using L = Lattice<Q>;
-  constexpr int V = Codec<S>::kV;
-  constexpr int NW = (7 + V - 1) / V;  // the words holding fields 0..6
-  const Nbr n = make_nbr(G, c);
-  C s[NW * V];
-#pragma unroll
-  for (int F = 0; F < NW * V; ++F) s[F] = C(0);
-#pragma unroll
-  for (int m = 0; m < NW; ++m) {
-#pragma unroll
-    for (int l = 0; l < Q; ++l) {
-      const S* src = f + read_index<Q, LAYOUT, S>(n, V * m, l);
-      C v[V];
-      if constexpr (V > 1)
-        Codec<S>::unpack(WordIO<S>::ldw_coh(src), v);
-      else
-        v[0] = Codec<S>::load_coh(src);
-#pragma unroll
-      for (int i = 0; i < V; ++i) s[V * m + i] += REP == kDEV ? C(L::w(l)) * v[i] : v[i];
-    }
-  }
-  s[0] = REP == kDEV ? log1p(s[0]) : log(s[0]);
-#pragma unroll
-  for (int F = 0; F < 7; ++F) aux[(int64_t)F * G.cells + c] = s[F];
-}
-
-template <int Q, class C>
-__device__ __forceinline__ void derivatives_coh(const Nbr& n, int64_t cells,
-                                                const C* __restrict__ aux, C inv2dx, C inv4dx,
-                                                C A[3], C D[3][6]) {
-  constexpr int dim = Lattice<Q>::kDim;
-#pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    if (k < dim) {
-      const uint32_t cp = n.at(k == 0, k == 1, k == 2);
-      const uint32_t cm = n.at(-(k == 0), -(k == 1), -(k == 2));
-      A[k] = (__ldcg(aux + cp) - __ldcg(aux + cm)) * inv2dx;
-#pragma unroll
-      for (int q = 0; q < 6; ++q) {
-        const C* plane = aux + (size_t)(1 + q) * (size_t)cells;
-        D[k][q] = (__ldcg(plane + cp) - __ldcg(plane + cm)) * inv4dx;
-      }
-    } else {
-      A[k] = C(0);
-#pragma unroll
-      for (int q = 0; q < 6; ++q) D[k][q] = C(0);
-    }
-  }
-}
-
-template <int Q, class S, class C, int REP, int LAYOUT, bool LAGW = false>
-__device__ __forceinline__ void collide_cell(const StepArgs<S, C>& a, int64_t c) {
-  using L = Lattice<Q>;
-  constexpr int dim = L::kDim;
-  const int64_t cells = a.G.cells;
-  constexpr int VW = Codec<S>::kV;  // fields per distribution word
-  const Nbr n = make_nbr(a.G, c);
-  C rt[kNF];
-#pragma unroll
-  for (int F = 0; F < kNF; ++F) rt[F] = C(0);
-#pragma unroll
-  for (int m = 0; m < kNF / VW; ++m) {
-#pragma unroll
-    for (int l = 0; l < Q; ++l) {
-      const S* src = a.fin + read_index<Q, LAYOUT, S>(n, VW * m, l);
-      C v[VW];
-      if constexpr (VW > 1)
-        Codec<S>::unpack(WordIO<S>::ldw_coh(src), v);
-      else
-        v[0] = Codec<S>::load_coh(src);
-#pragma unroll
-      for (int i = 0; i < VW; ++i) rt[VW * m + i] += REP == kDEV ? C(L::w(l)) * v[i] : v[i];
-    }
-  }
-  // reported at the end: a global write here would hold back the second
-  // pass's loads (see k_collide_w)
-  bool bad;
-  {
-    C chk = C(0);
-#pragma unroll
-    for (int F = 0; F < kNF; ++F) chk += rt[F];
-    bad = !isfinite(chk);
-  }
-  C A[3], D[3][6];
-  derivatives_coh<Q, C>(n, cells, a.aux, a.inv2dx, a.inv4dx, A, D);
-  C alpha, gm[6], K[6], V[3];
-  unpack<REP, C>(rt, alpha, gm, K, V);
-  C Sr[kNF];
-  bm_sources<C, dim>(alpha, gm, K, V, A, D, a.slicing, Sr);
-  add_fluid(a, alpha, gm, Sr);
-  if (!a.sources_on) {
-#pragma unroll
-    for (int F = 0; F < kNF; ++F) Sr[F] = C(0);
-  }
-  C rho[kNF];
-#pragma unroll
-  for (int F = 0; F < kNF; ++F) rho[F] = rt[F] + a.half_dt * Sr[F];
-  C Fl[6][3];
-  {
-    C alpha2, g2[6], K2[6], V2[3];
-    unpack<REP, C>(rho, alpha2, g2, K2, V2);
-    bm_flux<C, dim>(alpha2, g2, V2, A, D, Fl);
-  }
-  const C three_omega = C(3) * a.omega;
-  // FP64: the same weight-first form as k_collide, so a batched run stays
-  // bitwise equal to the run on its own context
-  constexpr bool kLeanRelax = sizeof(C) == 8 && REP == kABS;
-  if constexpr (VW == 1) {
-    // value by value, in k_collide's own expression form (the compiler
-    // contracts products into fused multiply-adds the same way in both)
-#pragma unroll
-    for (int F = 0; F < kNF; ++F) {
-      const C cf = a.omega * rho[F] + a.sigma * Sr[F];
-      C b[3] = {C(0), C(0), C(0)};
-      if (has_flux(F)) {
-#pragma unroll
-        for (int k = 0; k < dim; ++k) b[k] = three_omega * Fl[F - kK][k];
-      }
-      C v_[Q];
-#pragma unroll
-      for (int l = 0; l < Q; ++l) v_[l] = Codec<S>::load_coh(a.fin + read_index<Q, LAYOUT, S>(n, F, l));
+      for (int k = 0; k < 3; ++k) b[k] = flux(m, k);
 #pragma unroll
       for (int l = 0; l < Q; ++l) {
-        C t = kLeanRelax ? C(L::w(l)) * cf : cf;
-        if (has_flux(F)) {
+        C t = kWeighted ? C(L::w(l)) * cf[m] : cf[m];
+        if (fluxed(m)) {
 #pragma unroll
           for (int k = 0; k < dim; ++k) {
-            const C bk = kLeanRelax ? C(L::w(l)) * b[k] : b[k];
+            const C bk = kWeighted ? C(L::w(l) / kWb) * b[k] : b[k];
             if (L::c(l, k) > 0) t += bk;
             if (L::c(l, k) < 0) t -= bk;
           }
         }
-        const C out = REP == kDEV ? fma(a.omc, v_[l], t)
-                                  : (kLeanRelax ? fma(a.omc, v_[l], t)
-                                                : fma(a.omc, v_[l], C(L::w(l)) * t));
-        Codec<S>::store(a.fout + write_index<Q, LAYOUT, S>(n, F, l), out);
+        if (!kWeighted && REP == kABS) t *= C(L::w(l));
+        // Ping-pong: lanes past the last cell were clamped to it and write the
+        // same bytes as its own lanes, so every store can be unconditional.
+        S* dst = a.fout + write_index<Q, LAYOUT, S>(n, m, l);
+        const C out = fma(a.omc, vw[l], t);
+        if (LAYOUT == kPingPong)
+          Codec<S>::store(dst, out);
+        else
+          Codec<S>::store_if(dst, out, valid);
       }
-    }
-  } else {
+    } else if constexpr (!kLean) {
+      C b[V][3];
 #pragma unroll
-    for (int m = 0; m < kNF / VW; ++m) {
-      C cf[VW], b[VW][3];
+      for (int i = 0; i < V; ++i)
 #pragma unroll
-      for (int i = 0; i < VW; ++i) {
-        const int F = VW * m + i;
-        cf[i] = a.omega * rho[F] + a.sigma * Sr[F];
-#pragma unroll
-        for (int k = 0; k < 3; ++k) b[i][k] = has_flux(F) ? three_omega * Fl[F - kK][k] : C(0);
-      }
-      typename Codec<S>::W vw[Q];
+        for (int k = 0; k < 3; ++k) b[i][k] = flux(V * m + i, k);
 #pragma unroll
       for (int l = 0; l < Q; ++l) {
-        const S* src = a.fin + read_index<Q, LAYOUT, S>(n, VW * m, l);
-        vw[l] = WordIO<S>::ldw_coh(src);
-      }
-#pragma unroll
-      for (int l = 0; l < Q; ++l) {
-        C v[VW], out[VW];
+        C v[V], out[V];
         Codec<S>::unpack(vw[l], v);
 #pragma unroll
-        for (int i = 0; i < VW; ++i) {
-          C t = cf[i];
-          if (has_flux(VW * m + i)) {
+        for (int i = 0; i < V; ++i) {
+          C t = cf[V * m + i];
+          if (fluxed(V * m + i)) {
 #pragma unroll
             for (int k = 0; k < dim; ++k) {
               if (L::c(l, k) > 0) t += b[i][k];
@@ -991,13 +771,185 @@ __device__ __forceinline__ void collide_cell(const StepArgs<S, C>& a, int64_t c)
           }
           out[i] = REP == kDEV ? fma(a.omc, v[i], t) : fma(a.omc, v[i], C(L::w(l)) * t);
         }
-        S* dst = a.fout + write_index<Q, LAYOUT, S>(n, VW * m, l);
-        WordIO<S>::stw(dst, Codec<S>::pack(out));
+        S* dst = a.fout + write_index<Q, LAYOUT, S>(n, V * m, l);
+        if (LAYOUT == kPingPong)
+          WordIO<S>::stw(dst, Codec<S>::pack(out));
+        else
+          WordIO<S>::stw_if(dst, Codec<S>::pack(out), valid);
+      }
+    } else {
+      float2 c2[2], b[2][3];
+#pragma unroll
+      for (int p = 0; p < 2; ++p) {
+        const int F = V * m + 2 * p;
+        c2[p] = make_float2(cf[F], cf[F + 1]);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) b[p][k] = make_float2(flux(F, k), flux(F + 1, k));
+      }
+#pragma unroll
+      for (int l = 0; l < Q; ++l) {
+        float2 v[2];
+        unpack_pairs<S>(vw[l], v);
+#pragma unroll
+        for (int p = 0; p < 2; ++p) {
+          float2 t = c2[p];
+          if (fluxed(V * m + 2 * p) || fluxed(V * m + 2 * p + 1)) {
+#pragma unroll
+            for (int k = 0; k < dim; ++k) {
+              if (L::c(l, k) > 0) t = __fadd2_rn(t, b[p][k]);
+              if (L::c(l, k) < 0) t = __fadd2_rn(t, neg(b[p][k]));
+            }
+          }
+          v[p] = __ffma2_rn(pair(a.omc), v[p],
+                            REP == kDEV ? t : __fmul2_rn(pair((float)L::w(l)), t));
+        }
+        const float out[4] = {v[0].x, v[0].y, v[1].x, v[1].y};
+        S* dst = a.fout + write_index<Q, LAYOUT, S>(n, V * m, l);
+        if (LAYOUT == kPingPong)
+          WordIO<S>::stw(dst, Codec<S>::pack(out));
+        else
+          WordIO<S>::stw_if(dst, Codec<S>::pack(out), valid);
       }
     }
   }
-  if (LAGW) write_lagged<REP, C>(a.aux_out, cells, n.c, rho);
-  if (bad) atomicOr(a.flag, 1);
+  if (LAGW && valid) write_lagged<REP, C>(a.aux_out, cells, n.c, rho);
+  return bad;
+}
+
+// ---------------------------------------------------------------------------
+// One pass a launch, one thread per cell
+// ---------------------------------------------------------------------------
+// TPB threads a block, registers sized for MINB blocks per SM.
+template <int Q, class S, class C, int REP, int LAYOUT, bool HOLD, int SHIFT, bool LAGW, bool SUMS,
+          int TPB, int MINB>
+__global__ void __launch_bounds__(TPB, HOLD ? 1 : MINB) k_collide(const StepArgs<S, C> a) {
+  const int64_t cell = (int64_t)blockIdx.x * TPB + threadIdx.x;
+  const bool valid = cell < a.G.cells;
+  const Nbr n = make_nbr(a.G, valid ? cell : a.G.cells - 1);
+  if (collide_body<Q, S, C, REP, LAYOUT, SHIFT, HOLD, SUMS, LAGW, false, false>(a, n, valid, Plain()))
+    atomicOr(a.flag, 1);
+}
+
+template <int Q, class S, class C, int REP, int LAYOUT>
+__global__ void __launch_bounds__(256) k_aux(const S* __restrict__ f, C* __restrict__ aux, C* sums,
+                                             Grid G) {
+  const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (c < G.cells)
+    aux_body<Q, S, C, REP, LAYOUT, kKeep>(f, aux, sums, G.cells, make_nbr(G, c), true);
+}
+
+// ---------------------------------------------------------------------------
+// k_step: the moment pass and the collide pass in one launch (SYNC)
+// ---------------------------------------------------------------------------
+// As two launches the alpha and gamma words cross HBM twice: the moment pass
+// reads 608 of the 1216 bytes of a cell (FP32, D3Q19), and by the time the
+// collide pass comes to them they have left the L2. Here both passes go
+// through the lattice together, the moment pass a short way ahead, so that the
+// collide pass finds those words in the L2 (256 x 256 x 24, ncu: 2631 DRAM
+// bytes a cell-step, against 2460 + 636 in two launches), and takes their sums
+// from the planes: its pass 1 reads only the other half.
+//
+// Work items are warps of 32 cells (one tile), claimed from a counter: the
+// moment pass of a tile and the collide pass of one a few units behind it
+// (schedule.h holds the list). A collide tile sums its words first and then
+// waits until the moment pass of every unit up to that of its last neighbour
+// is complete (one counter a unit). Items are claimed in list order, moment
+// tiles never wait, and a collide tile waits only for moment tiles of items
+// before its own, so the first unfinished item always runs: no wait can outlast
+// the work before it. Every wait is bounded all the same (bit 1 of the flag
+// after ~2 s).
+//
+// A cell's moment tile reads what only the cell's own collide tile writes (in
+// place) or a buffer that the launch does not write (ping-pong).
+//
+// us a step, D3Q19 FP32, blocks of 64 threads x 4, against two launches (same
+// arithmetic, same blocks): 64^3 112 / 134, 128^3 855 / 955, 256^3 6885 / 7690;
+// 149 x 101 x 67 in place 441 / 495. Bound by HBM at 0.93 of the copy rate and by
+// the chain of loads of a warp (claim, moment words, pass 1, planes, pass 2).
+// What did not help: claiming the next item early or publishing the moments
+// late (7107: the passes move apart), an L2 prefetch a unit ahead (6913), the
+// words of pass 1 staged in shared memory (7557), 10 or 12 warps per SM (7608:
+// the words no longer stay in the L2). 16-bit storage gains nothing (4261
+// against 4290: it waits on its conversions, not on HBM), and D2Q9 loses (240
+// against 227), so both keep two launches; so does FP64, bound by its operations.
+__device__ __forceinline__ unsigned ld_acquire(const unsigned* p) {
+  unsigned v;
+  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ void red_release(unsigned* p, unsigned v) {
+  asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+__device__ __forceinline__ uint64_t step_clock_ns() {
+  uint64_t t;
+  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+  return t;
+}
+
+template <int Q, class S, class C, int REP, int LAYOUT, int SHIFT, int TPB, int MINB>
+__global__ void __launch_bounds__(TPB, MINB) k_step(const StepArgs<S, C> a, C* aux, C* sums,
+                                                     const Schedule s) {
+  constexpr uint64_t kLimitNs = 2000000000ull;
+  const uint32_t lane = threadIdx.x & 31u;
+  const int64_t cells = a.G.cells;
+  unsigned done_to = 0;  // moment units at list positions [0, done_to) are complete
+  for (;;) {
+    uint32_t item = 0;
+    if (lane == 0) item = atomicAdd(s.cnt, 1u);
+    item = __shfl_sync(0xffffffffu, item, 0);
+    if (item >= s.items) break;
+    const Item t = item_at(s, item);
+    uint32_t tile, need;
+    if (t.pos < s.units) {
+      if (moment_tile(s, t, tile)) {
+        const int64_t cell = (int64_t)tile * 32 + lane;
+        const bool valid = cell < cells;
+        aux_body<Q, S, C, REP, LAYOUT, LAYOUT == kPingPong ? kKeep : kCoherent>(
+            a.fin, aux, sums, cells, make_nbr(a.G, valid ? cell : cells - 1), valid);
+      }
+      __syncwarp();
+      if (lane == 0) {
+        red_release(s.cnt + 1 + t.pos, 1u);
+        if (t.slot == 0) s.cnt_next[1 + t.pos] = 0u;
+        if (item == 0) s.cnt_next[0] = 0u;
+      }
+    }
+    if (!collide_tile(s, t, tile, need)) continue;
+    const int64_t cell = (int64_t)tile * 32 + lane;
+    const bool valid = cell < cells;
+    const Nbr n = make_nbr(a.G, valid ? cell : cells - 1);
+    bool late = false;
+    auto before_planes = [&] {
+      uint64_t t0 = 0;
+      while (done_to <= need) {
+        const unsigned u = done_to + lane;
+        const bool ok = u > need || ld_acquire(s.cnt + 1 + u) >= s.slots;
+        const unsigned open = ~__ballot_sync(0xffffffffu, ok);
+        done_to += open ? (unsigned)__ffs((int)open) - 1u : 32u;
+        if (done_to > need) {
+          done_to = need + 1u;  // the lanes past it have looked at nothing
+          break;
+        }
+        if (open) {
+          const uint64_t now = step_clock_ns();
+          if (t0 == 0) t0 = now;
+          if (__shfl_sync(0xffffffffu, (unsigned)(now - t0 > kLimitNs), 0)) {
+            late = true;
+            break;
+          }
+          __nanosleep(20);
+        }
+      }
+      __syncwarp();
+    };
+    const bool bad = collide_body<Q, S, C, REP, LAYOUT, SHIFT, false, true, false, false, true>(
+        a, n, valid, Hooked<decltype(before_planes)>{before_planes});
+    if (bad) atomicOr(a.flag, 1);
+    if (late) {
+      if (lane == 0) atomicOr(a.flag, 2);
+      break;
+    }
+  }
 }
 
 // ---------------------------------------------------------------------------
