@@ -44,19 +44,22 @@ LBNR_VARIANTS(19, 8, 0, {0, 1, false, 0, 0, 0}, {1, 1, false, 2, 1, 32})
 // layout they ran at half the speed and are not offered.) The re-read forms
 // come in three block shapes: 128 threads x 3 blocks per SM (168 registers),
 // 64 x 4 and 128 x 2 (255 registers, 8 warps per SM: fewer cells resident,
-// so more of the update pass's re-read stays in L2).
+// so more of the update pass's re-read stays in L2). Form 0, what a context
+// runs until another one is chosen, is for D3Q19 the one that is fastest over
+// 16^3 to 256^3: 64 x 4 for FP32 (us a step at 128^3: 855, bulk-copy-fed 1071;
+// LAG at 160^3: 1503, 1745), 128 x 3 for 16 bits (256^3 collide: 3.48 ms, 3.88).
 LBNR_VARIANTS(3, 4, 1, {1, 1, false, 8, 4, 32}, {0, 1, true, 0, 0, 0}, {0, 1, false, 0, 0, 0},
               {0, 1, false, 0, 0, 0, 64, 4})
 LBNR_VARIANTS(9, 4, 1, {1, 1, false, 4, 2, 32}, {0, 1, true, 0, 0, 0}, {0, 1, false, 0, 0, 0},
               {0, 1, false, 0, 0, 0, 64, 4})
-LBNR_VARIANTS(19, 4, 2, {1, 1, false, 4, 1, 32}, {1, 1, false, 5, 1, 32}, {0, 1, false, 0, 0, 0},
-              {0, 1, false, 0, 0, 0, 64, 4}, {0, 1, false, 0, 0, 0, 128, 2})
+LBNR_VARIANTS(19, 4, 1, {0, 1, false, 0, 0, 0, 64, 4}, {0, 1, false, 0, 0, 0},
+              {0, 1, false, 0, 0, 0, 128, 2}, {1, 1, false, 4, 1, 32}, {1, 1, false, 5, 1, 32})
 LBNR_VARIANTS(3, 2, 1, {1, 1, false, 8, 4, 32}, {0, 1, true, 0, 0, 0}, {0, 1, false, 0, 0, 0},
               {0, 1, false, 0, 0, 0, 64, 4})
 LBNR_VARIANTS(9, 2, 1, {1, 1, false, 8, 2, 32}, {0, 1, true, 0, 0, 0}, {0, 1, false, 0, 0, 0},
               {0, 1, false, 0, 0, 0, 64, 4})
-LBNR_VARIANTS(19, 2, 1, {1, 1, false, 8, 1, 32}, {0, 1, false, 0, 0, 0},
-              {0, 1, false, 0, 0, 0, 64, 4}, {0, 1, false, 0, 0, 0, 128, 2})
+LBNR_VARIANTS(19, 2, 0, {0, 1, false, 0, 0, 0}, {0, 1, false, 0, 0, 0, 64, 4},
+              {0, 1, false, 0, 0, 0, 128, 2}, {1, 1, false, 8, 1, 32})
 #undef LBNR_VARIANTS
 
 inline int sm_count() {
@@ -149,13 +152,15 @@ struct Impl {
   static cudaError_t launch_generic(const LaunchCtx& L, const StepArgs<S, C>& a, bool one_launch) {
     constexpr VariantSpec x = VT::v[VI];
     static_assert(x.P == 1, "one thread per cell");
-    constexpr int TPB = x.tpb > 0 ? x.tpb : 128;
     // The default shape, 128 threads sized for 3 blocks per SM, takes 2 where
     // it would spill: word by word at the odd AA step, which holds a field
     // group's Q words and reads and writes at neighbours, and in FP64 with the
-    // lagged-field writes.
-    constexpr int MINB = x.minb > 0 ? x.minb : (Codec<S>::kV > 1 && LAYOUT == kAAOdd ? 2 : 3);
-    constexpr int LAGMINB = Codec<S>::kV > 1 ? MINB : 2;
+    // lagged-field writes. FP64 takes the same in blocks of 64: bound by its
+    // operations, it waits for the SM with the most cells.
+    constexpr bool kWords = Codec<S>::kV > 1;
+    constexpr int TPB = x.tpb > 0 ? x.tpb : kWords ? 128 : 64;
+    constexpr int MINB = x.minb > 0 ? x.minb : kWords ? (LAYOUT == kAAOdd ? 2 : 3) : 6;
+    constexpr int LAGMINB = kWords ? MINB : 4;
     return launch_form<LAYOUT, 0, x.hold, TPB, MINB, LAGMINB>(L, a, one_launch);
   }
 
