@@ -218,18 +218,21 @@ int lbnr_set_shift(lbnr_ctx* ctx, double bx, double by, double bz);
 int lbnr_set_shift_field(lbnr_ctx* ctx, const double* beta);
 
 /* Launch forms of the collide kernel available for this context's set and
- * storage (all give the same results within rounding; every form runs one
- * thread per cell): their number, a short name, and the selection (default
- * 0). Used by the autotuner. Names: "P1-hold" / "P1-reread" (distributions
- * held in registers between the moment and update passes, or read again),
- * with a suffix "-<t>x<b>" for blocks of t threads sized for b blocks per SM
- * (no suffix: 128 x 3); "tma-p1-nc<c>-k<k>-t32" (persistent, fed by bulk
- * copies of whole 32-cell tiles, c consumer warps with k stages each). The
- * bulk-copy-fed forms read each tile's own cells only; at the odd step of the
- * in-place pattern a register form runs in their place. */
+ * storage (all give the same results within rounding): their number, a short
+ * name, and the selection (default: form 0, for small FP64 ping-pong lattices
+ * "lanes16" or "lanes8"; lbnr_variant returns it, -1 for NULL). Used by the
+ * autotuner. Names: "P1-hold" / "P1-reread" (distributions held in registers
+ * between the moment and update passes, or read again), with a suffix
+ * "-<t>x<b>" for blocks of t threads sized for b blocks per SM (no suffix: 128
+ * x 3, FP64 64 x 6); "tma-p1-nc<c>-k<k>-t32" (persistent, fed by bulk copies of
+ * whole 32-cell tiles, c consumer warps with k stages each); "lanes<n>" (FP64:
+ * n lanes share a cell; in place form 0 runs instead). The others run one
+ * thread per cell. The bulk-copy-fed forms read each tile's own cells only; at
+ * the odd step of the in-place pattern a register form runs in their place. */
 int lbnr_num_variants(const lbnr_ctx* ctx);
 const char* lbnr_variant_name(const lbnr_ctx* ctx, int variant);
 int lbnr_set_variant(lbnr_ctx* ctx, int variant);
+int lbnr_variant(const lbnr_ctx* ctx);
 
 /* Steps taken since lbnr_init; Q of the velocity set; the streaming pattern
  * chosen (LBNR_STREAM_PINGPONG or LBNR_STREAM_AA). */

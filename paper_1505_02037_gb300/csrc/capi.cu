@@ -453,6 +453,8 @@ int lbnr_create(const lbnr_grid* grid, int vset, double tau, double dx, double d
   L.beta[0] = L.beta[1] = L.beta[2] = 0;
   L.shift_on = 0;
   L.beta_field = nullptr;
+  L.pingpong = streaming == LBNR_STREAM_PINGPONG ? 1 : 0;
+  c->variant = ops->default_variant(L);
   // zero everything once: the padding cells of the last tile must hold finite values
   cudaError_t e = cudaMemsetAsync(c->base, 0, Ly.total, c->st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(c->st);
@@ -756,6 +758,8 @@ int lbnr_set_variant(lbnr_ctx* c, int v) {
   }
   return LBNR_OK;
 }
+
+int lbnr_variant(const lbnr_ctx* c) { return c ? c->variant : -1; }
 
 int64_t lbnr_steps_done(const lbnr_ctx* c) { return c ? c->steps : -1; }
 int lbnr_q(const lbnr_ctx* c) { return c ? c->Q : 0; }

@@ -43,6 +43,7 @@ struct LaunchCtx {
   // The work list of the step that runs both passes in one launch, with the
   // counters of this step (units = 0: one pass a launch).
   Schedule sched;
+  int pingpong;  // 0: in place
 };
 
 // layout: 0 ping-pong, 1 AA at even step, 2 AA at odd step
@@ -65,6 +66,8 @@ struct Ops {
   cudaError_t (*lag_to64)(const LaunchCtx&, const void* aux, double* out);
   // whether step() of this variant runs the moment pass itself
   bool (*fused)(const LaunchCtx&, int variant);
+  // the variant a context starts with
+  int (*default_variant)(const LaunchCtx&);
 };
 
 // One getter per (velocity set, storage), each in its own translation unit

@@ -5,6 +5,7 @@
 
 #include "collide_tma.cuh"
 #include "kernels.cuh"
+#include "lanes.cuh"
 
 namespace lbnr {
 
@@ -17,10 +18,12 @@ namespace lbnr {
 //         warps and NC K shared-memory stages of one 32-cell tile; local
 //         reads only, so at the odd AA step it hands over to the form named
 //         by `fallback`.
+// kind 2: NC lanes per cell (lanes.cuh), FP64 and ping-pong; in place the form
+//         named by `fallback` runs.
 struct VariantSpec {
   int kind, P;
   bool hold;
-  int nc, k, tc;  // consumer warps, stages per warp, cells per tile (kind 1)
+  int nc, k, tc;  // consumer warps, stages per warp, cells per tile (kind 1); lanes (2)
   int tpb, minb;  // kind 0, word forms: threads per block and the blocks per SM the
                   // registers are sized for (0: 128 and 3)
 };
@@ -36,9 +39,9 @@ struct VariantTable;
     static constexpr int fallback = FALLBACK_;               \
   };
 // FP64 storage (FP64 arithmetic)
-LBNR_VARIANTS(3, 8, 0, {0, 1, true, 0, 0, 0}, {1, 1, false, 8, 1, 32})
-LBNR_VARIANTS(9, 8, 0, {0, 1, false, 0, 0, 0}, {1, 1, false, 4, 1, 32})
-LBNR_VARIANTS(19, 8, 0, {0, 1, false, 0, 0, 0}, {1, 1, false, 2, 1, 32})
+LBNR_VARIANTS(3, 8, 0, {0, 1, true, 0, 0, 0}, {1, 1, false, 8, 1, 32}, {2, 1, false, 16, 0, 0}, {2, 1, false, 8, 0, 0})
+LBNR_VARIANTS(9, 8, 0, {0, 1, false, 0, 0, 0}, {1, 1, false, 4, 1, 32}, {2, 1, false, 16, 0, 0}, {2, 1, false, 8, 0, 0})
+LBNR_VARIANTS(19, 8, 0, {0, 1, false, 0, 0, 0}, {1, 1, false, 2, 1, 32}, {2, 1, false, 16, 0, 0}, {2, 1, false, 8, 0, 0})
 // FP32 and 16-bit storage: one lane per cell, word by word. (Forms with two
 // lanes per cell split a word's fields between the lanes; on the word
 // layout they ran at half the speed and are not offered.) The re-read forms
@@ -95,7 +98,9 @@ struct Impl {
     static char buf[8][48];
     if (v < 0 || v >= VT::n || v >= 8) return "?";
     const VariantSpec& x = VT::v[v];
-    if (x.kind == 0 && x.tpb > 0)
+    if (x.kind == 2)
+      snprintf(buf[v], sizeof(buf[v]), "lanes%d", x.nc);
+    else if (x.kind == 0 && x.tpb > 0)
       snprintf(buf[v], sizeof(buf[v]), "P%d%s-%dx%d", x.P, x.hold ? "-hold" : "-reread", x.tpb,
                x.minb);
     else if (x.kind == 0)
@@ -109,10 +114,19 @@ struct Impl {
   static constexpr bool kOneLaunch = Q == 19 && sizeof(S) == 4;
   // Whether the step of this variant runs the moment pass itself.
   static bool fused(const LaunchCtx& L, int variant) {
+    const VariantSpec& x = VT::v[variant >= 0 && variant < VT::n ? variant : 0];
+    if (x.kind == 2 && L.pingpong && !L.shift_on && !L.beta_field) return true;
     if (!kOneLaunch || L.sched.units == 0 || L.aux_out) return false;
     if (L.shift_on || L.beta_field) return true;
-    const VariantSpec& x = VT::v[variant >= 0 && variant < VT::n ? variant : 0];
     return x.kind == 0 && !x.hold;
+  }
+
+  // The form a context starts with: 0, or several lanes per cell for FP64
+  // lattices too small to fill the schedulers with a thread per cell.
+  static int default_variant(const LaunchCtx& L) {
+    for (int v = 0; v < VT::n; ++v)
+      if (VT::v[v].kind == 2 && L.pingpong && VT::v[v].nc == lanes_for<Q>(L.cells)) return v;
+    return 0;
   }
 
   template <int LAYOUT, int SHIFT, int TPB, int MINB>
@@ -199,7 +213,19 @@ struct Impl {
 
   template <int LAYOUT, int VI>
   static cudaError_t launch_variant(const LaunchCtx& L, const StepArgs<S, C>& a) {
-    if constexpr (VT::v[VI].kind == 1) {
+    if constexpr (VT::v[VI].kind == 2) {
+      if constexpr (LAYOUT == kPingPong) {
+        constexpr int NL = VT::v[VI].nc;
+        const unsigned grid = grid_for(L.cells, 32 / NL);
+        if (a.aux_out)
+          k_lanes<Q, NL, true><<<grid, 32, 0, L.st>>>(a);
+        else
+          k_lanes<Q, NL, false><<<grid, 32, 0, L.st>>>(a);
+        return cudaGetLastError();
+      } else {
+        return launch_generic<LAYOUT, VT::fallback>(L, a, false);
+      }
+    } else if constexpr (VT::v[VI].kind == 1) {
       if constexpr (LAYOUT == kAAOdd)
         return launch_generic<LAYOUT, VT::fallback>(L, a, false);
       else
@@ -386,7 +412,7 @@ struct Impl {
   static const Ops* ops() {
     static const Ops o = {VT::n,     &variant_name, &step,          &aux,       &init,
                           &sum64,    &correct64,    &constraints64, &get_plane, &set_plane,
-                          &get_cells, &lag_from64,  &lag_to64, &fused};
+                          &get_cells, &lag_from64,  &lag_to64, &fused, &default_variant};
     return &o;
   }
 };

@@ -97,6 +97,7 @@ def library(path: str | None = None):
     L.lbnr_variant_name.argtypes = [vp, ctypes.c_int]
     L.lbnr_variant_name.restype = ctypes.c_char_p
     L.lbnr_set_variant.argtypes = [vp, ctypes.c_int]
+    L.lbnr_variant.argtypes = [vp]
     L.lbnr_set_fluid.argtypes = [vp, ctypes.c_double, ctypes.c_double, ctypes.c_double]
     L.lbnr_set_shift.argtypes = [vp, ctypes.c_double, ctypes.c_double, ctypes.c_double]
     L.lbnr_set_shift_field.argtypes = [vp, vp]
@@ -420,7 +421,7 @@ class Lattice:
         self.dt = float(dx if dt is None else dt)
         self.ctx = lbnr_create(self.grid, self.vset, self.tau, self.dx, self.dt, o)
         self.streaming = library().lbnr_streaming(self.ctx)
-        self.variant = 0
+        self.variant = library().lbnr_variant(self.ctx)
 
     def init(self, fields):
         a = fields if not isinstance(fields, np.ndarray) else np.ascontiguousarray(
