@@ -709,13 +709,12 @@ int lbnr_batch_get_distributions(lbnr_batch* b, int run, double* out) {
   L.pstride = h.G.pstride;
   L.st = b->st;
   const size_t cells = (size_t)h.G.cells;
-  for (int F = 0; F < 16; ++F)
-    for (int l = 0; l < h.q; ++l) {
-      double* plane = b->d_stage + (size_t)((F * h.q + l) % 16) * cells;
-      BTRY(b, o->get_plane(L, 0, h.f[done & 1], F, l, plane));
-      BTRY(b, cudaMemcpyAsync(out + (size_t)(F * h.q + l) * cells, plane, sizeof(double) * cells,
-                              cudaMemcpyDeviceToHost, b->st));
-    }
+  // sixteen planes at a time through the staging area
+  for (int p = 0; p < 16 * h.q; p += 16) {
+    BTRY(b, o->get_planes(L, 0, h.f[done & 1], p, 16, b->d_stage));
+    BTRY(b, cudaMemcpyAsync(out + (size_t)p * cells, b->d_stage, sizeof(double) * 16 * cells,
+                            cudaMemcpyDeviceToHost, b->st));
+  }
   BTRY(b, cudaStreamSynchronize(b->st));
   return LBNR_OK;
 }

@@ -56,7 +56,9 @@ struct Ops {
   cudaError_t (*sum64)(const LaunchCtx&, int layout, const void* f, int64_t* nblocks);
   cudaError_t (*correct64)(const LaunchCtx&);
   cudaError_t (*constraints64)(const LaunchCtx&, int64_t* nblocks);
-  cudaError_t (*get_plane)(const LaunchCtx&, int layout, const void* f, int F, int l, double* out);
+  // planes [p0, p0 + np) of the standard order F Q + l
+  cudaError_t (*get_planes)(const LaunchCtx&, int layout, const void* f, int p0, int np,
+                            double* out);
   cudaError_t (*set_plane)(const LaunchCtx&, int layout, void* f, int F, int l, const double* in);
   cudaError_t (*get_cells)(const LaunchCtx&, int layout, const void* f, int64_t n,
                            const int64_t* idx, double* out);

@@ -364,14 +364,14 @@ struct Impl {
     return cudaGetLastError();
   }
 
-  static cudaError_t get_plane(const LaunchCtx& L, int layout, const void* f, int F, int l,
-                               double* out) {
+  static cudaError_t get_planes(const LaunchCtx& L, int layout, const void* f, int p0, int np,
+                                double* out) {
     const Grid G = make_grid(L.nx, L.ny, L.nz, L.cells, L.pstride);
-    const unsigned grid = grid_for(L.cells, 256);
+    const dim3 grid(grid_for(L.cells, 256), (unsigned)np);
     const S* fp = static_cast<const S*>(f);
-    if (layout == kPingPong) k_get_plane<Q, S, REP, kPingPong><<<grid, 256, 0, L.st>>>(fp, out, G, F, l);
-    else if (layout == kAAEven) k_get_plane<Q, S, REP, kAAEven><<<grid, 256, 0, L.st>>>(fp, out, G, F, l);
-    else k_get_plane<Q, S, REP, kAAOdd><<<grid, 256, 0, L.st>>>(fp, out, G, F, l);
+    if (layout == kPingPong) k_get_planes<Q, S, REP, kPingPong><<<grid, 256, 0, L.st>>>(fp, out, G, p0);
+    else if (layout == kAAEven) k_get_planes<Q, S, REP, kAAEven><<<grid, 256, 0, L.st>>>(fp, out, G, p0);
+    else k_get_planes<Q, S, REP, kAAOdd><<<grid, 256, 0, L.st>>>(fp, out, G, p0);
     return cudaGetLastError();
   }
 
@@ -411,7 +411,7 @@ struct Impl {
 
   static const Ops* ops() {
     static const Ops o = {VT::n,     &variant_name, &step,          &aux,       &init,
-                          &sum64,    &correct64,    &constraints64, &get_plane, &set_plane,
+                          &sum64,    &correct64,    &constraints64, &get_planes, &set_plane,
                           &get_cells, &lag_from64,  &lag_to64, &fused, &default_variant};
     return &o;
   }

@@ -1364,19 +1364,23 @@ __global__ void __launch_bounds__(128) k_constraints64(const double* __restrict_
   }
 }
 
-// Plane transfer between the FP64 standard layout and the stored state.
+// Plane transfers between the FP64 standard layout and the stored state: planes
+// [p0, p0 + gridDim.y) of the standard order F Q + l in one launch.
 template <int Q, class S, int REP, int LAYOUT>
-__global__ void k_get_plane(const S* __restrict__ f, double* __restrict__ out, Grid G, int F, int l) {
+__global__ void k_get_planes(const S* __restrict__ f, double* __restrict__ out, Grid G, int p0) {
   using L = Lattice<Q>;
   const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= G.cells) return;
+  const int F = (p0 + (int)blockIdx.y) / Q, l = (p0 + (int)blockIdx.y) % Q;
   const Nbr n = make_nbr(G, c);
-  const double v = (double)Codec<S>::load_keep(f + read_index<Q, LAYOUT, S>(n, F, l));
-  double w = 0;
+  double v = 0, w = 0;
 #pragma unroll
   for (int ll = 0; ll < Q; ++ll)
-    if (ll == l) w = L::w(ll);
-  out[c] = REP == kDEV ? w * (v + flat_value(F)) : v;
+    if (ll == l) {
+      w = L::w(ll);
+      v = (double)Codec<S>::load_keep(f + read_index<Q, LAYOUT, S>(n, F, ll));
+    }
+  out[(int64_t)blockIdx.y * G.cells + c] = REP == kDEV ? w * (v + flat_value(F)) : v;
 }
 
 template <int Q, class S, int REP, int LAYOUT>
