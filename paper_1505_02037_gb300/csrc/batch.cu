@@ -290,7 +290,7 @@ struct lbnr_batch {
   unsigned* d_bar = nullptr;
   int* d_status = nullptr;
   int* d_flag = nullptr;
-  double* d_stage = nullptr;  // 16 x max cells FP64 (init, transfers)
+  double* d_stage = nullptr;  // 17 x max cells FP64 (init, transfers)
   int64_t max_cells = 0;
   int grid = 0, block = 256, form = 0;
   std::vector<Assign> work;
@@ -516,7 +516,7 @@ int lbnr_batch_create(int nruns, const lbnr_run_desc* runs, const lbnr_batch_opt
                : (((size_t)9 * cells * cb + 255) & ~(size_t)255);
   }
   const size_t stage_off = off;
-  off += ((size_t)16 * b->max_cells * 8 + 255) & ~(size_t)255;
+  off += ((size_t)17 * b->max_cells * 8 + 255) & ~(size_t)255;
   b->bytes = off;
   cudaError_t e = cudaMalloc(&b->base, off);
   if (e != cudaSuccess) {
@@ -603,6 +603,7 @@ int lbnr_batch_init(lbnr_batch* b, int run, const double* fields) {
   L.slicing = d.slicing;
   L.sources_on = b->opts.sources_on ? 1 : 0;
   L.macro = b->d_stage;
+  L.aux64 = b->d_stage + 16 * cells;
   L.flag = b->d_status + run;
   L.st = b->st;
   const Ops* o = ops_for_run(d.vset, b->opts.storage);

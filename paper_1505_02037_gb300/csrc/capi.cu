@@ -620,9 +620,10 @@ int lbnr_moments(lbnr_ctx* c, double* out) {
   c->L.fluid_P_now = fluid_pressure_now(c);
   CUDA_TRY(c, c->ops->sum64(c->L, layout_now(c), state_now(c), &nb));
   if (lagged(c)) CUDA_TRY(c, c->ops->lag_to64(c->L, c->aux[c->steps & 1], nullptr));
-  CUDA_TRY(c, c->ops->correct64(c->L));
-  CUDA_TRY(c, copy_fields(c, out, c->L.macro, sizeof(double) * 16 * (size_t)c->L.cells,
-                          cudaMemcpyDeviceToHost));
+  const size_t nb_out = sizeof(double) * 16 * (size_t)c->L.cells;
+  double* const direct = static_cast<double*>(mapped(out, nb_out));
+  CUDA_TRY(c, c->ops->correct64(c->L, direct ? direct : c->L.macro));
+  if (!direct) CUDA_TRY(c, cudaMemcpyAsync(out, c->L.macro, nb_out, cudaMemcpyDeviceToHost, c->st));
   int flag = 0;
   int rc = read_flag(c, &flag);
   if (rc) return rc;
@@ -636,7 +637,7 @@ int lbnr_constraints(lbnr_ctx* c, double* out) {
   c->L.fluid_P_now = fluid_pressure_now(c);
   CUDA_TRY(c, c->ops->sum64(c->L, layout_now(c), state_now(c), &nbs));
   if (lagged(c)) CUDA_TRY(c, c->ops->lag_to64(c->L, c->aux[c->steps & 1], nullptr));
-  CUDA_TRY(c, c->ops->correct64(c->L));
+  CUDA_TRY(c, c->ops->correct64(c->L, c->L.macro));
   CUDA_TRY(c, c->ops->constraints64(c->L, &nbc));
   CUDA_TRY(c, reduce_final(c->L.partials, nbc, nbs, c->L.cells, c->L.out22, c->st));
   CUDA_TRY(c, cudaMemcpyAsync(out, c->L.out22, sizeof(double) * 22, cudaMemcpyDeviceToHost, c->st));

@@ -54,7 +54,7 @@ struct Ops {
   cudaError_t (*aux)(const LaunchCtx&, int layout, const void* f);
   cudaError_t (*init)(const LaunchCtx&, void* f);  // from macro, standard layout
   cudaError_t (*sum64)(const LaunchCtx&, int layout, const void* f, int64_t* nblocks);
-  cudaError_t (*correct64)(const LaunchCtx&);
+  cudaError_t (*correct64)(const LaunchCtx&, double* out);  // out: macro or [16][cells] elsewhere
   cudaError_t (*constraints64)(const LaunchCtx&, int64_t* nblocks);
   // planes [p0, p0 + np) of the standard order F Q + l
   cudaError_t (*get_planes)(const LaunchCtx&, int layout, const void* f, int p0, int np,

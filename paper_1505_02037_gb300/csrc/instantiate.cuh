@@ -328,7 +328,11 @@ struct Impl {
     for (int k = 0; k < 3; ++k) a.beta[k] = L.beta[k];
     a.shift_on = L.shift_on;
     a.beta_field = L.beta_field;
-    k_init<Q, S, REP><<<grid_for(L.cells, 128), 128, 0, L.st>>>(a);
+    a.lnalpha = L.aux64;
+    k_log<<<grid_for(L.cells, 256), 256, 0, L.st>>>(L.macro, L.aux64, L.cells);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    k_init<Q, S, REP><<<grid_for(L.cells, 64), 64, 0, L.st>>>(a);
     return cudaGetLastError();
   }
 
@@ -346,10 +350,10 @@ struct Impl {
     return cudaGetLastError();
   }
 
-  static cudaError_t correct64(const LaunchCtx& L) {
+  static cudaError_t correct64(const LaunchCtx& L, double* out) {
     const Grid G = make_grid(L.nx, L.ny, L.nz, L.cells, L.pstride);
     k_correct64<Q><<<grid_for(L.cells, 128), 128, 0, L.st>>>(
-        L.macro, L.aux64, G, 1.0 / (2.0 * L.dx), 1.0 / (4.0 * L.dx), 0.5 * L.dt, L.slicing,
+        L.macro, out, L.aux64, G, 1.0 / (2.0 * L.dx), 1.0 / (4.0 * L.dx), 0.5 * L.dt, L.slicing,
         L.sources_on, L.clock ? L.fluid_P_now : 0.0, L.shift_on ? L.beta[0] : 0.0,
         L.shift_on ? L.beta[1] : 0.0, L.shift_on ? L.beta[2] : 0.0, L.beta_field);
     return cudaGetLastError();

@@ -958,6 +958,7 @@ __global__ void __launch_bounds__(TPB, MINB) k_step(const StepArgs<S, C> a, C* a
 template <class S>
 struct Init64Args {
   const double* fields;  // [16][cells]
+  const double* lnalpha; // [cells]
   S* f;                  // standard layout
   int* flag;
   Grid G;
@@ -969,11 +970,23 @@ struct Init64Args {
   const double* beta_field;  // static shift field [3][cells] or nullptr
 };
 
+// ln alpha of the initial fields, once per cell: k_init differentiates it.
+static __global__ void __launch_bounds__(256) k_log(const double* __restrict__ alpha,
+                                                    double* __restrict__ out, int64_t cells) {
+  const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (c < cells) out[c] = log(alpha[c]);
+}
+
 // Shifted equilibrium: f = f_eq(rho0) - (dt/2) w_l S(rho0), A and D from rho0.
+// Bound by its FP64 operations, so logarithms come from k_log (six of them a
+// cell otherwise), the fluxes carry 3 w_l from the start, and a value is
+// w_l (rho - dt S / 2) plus at most three of them: lbnr_init at 256^3 FP32 56 ms,
+// 74 before (10 of them the copy from the host).
 template <int Q, class S, int REP>
-__global__ void __launch_bounds__(128) k_init(const Init64Args<S> a) {
+__global__ void __launch_bounds__(64) k_init(const Init64Args<S> a) {
   using L = Lattice<Q>;
   constexpr int dim = L::kDim;
+  constexpr double kWb = REP == kDEV ? 1.0 : L::w(Q - 1);  // the weight that fluxes carry
   const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= a.G.cells) return;
   const int64_t cells = a.G.cells;
@@ -987,7 +1000,7 @@ __global__ void __launch_bounds__(128) k_init(const Init64Args<S> a) {
     if (k < dim) {
       const int64_t cp = n.at(k == 0, k == 1, k == 2);
       const int64_t cm = n.at(-(k == 0), -(k == 1), -(k == 2));
-      A[k] = (log(a.fields[cp]) - log(a.fields[cm])) * a.inv2dx;
+      A[k] = (a.lnalpha[cp] - a.lnalpha[cm]) * a.inv2dx;
 #pragma unroll
       for (int q = 0; q < 6; ++q)
         D[k][q] = (a.fields[(int64_t)(1 + q) * cells + cp] - a.fields[(int64_t)(1 + q) * cells + cm]) *
@@ -1011,32 +1024,39 @@ __global__ void __launch_bounds__(128) k_init(const Init64Args<S> a) {
   if (!a.sources_on)
     for (int F = 0; F < kNF; ++F) Sr[F] = 0;
   double Fl[6][3], Fv[3][3];
-  bm_flux<double, dim>(alpha, gm, V, A, D, Fl);
-  if (a.shift_on) shift_flux_k<double, dim>(sb, K, Fl);
-  if (a.beta_field) shift_field_vflux<double, dim>(gm, V, sb, sB, Fv);
+  constexpr double fs = 3.0 * kWb;
+  bm_flux<double, dim>(alpha * fs, gm, V, A, D, Fl);
+  if (a.shift_on) {
+    const double bs[3] = {fs * sb[0], fs * sb[1], fs * sb[2]};
+    shift_flux_k<double, dim>(bs, K, Fl);
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+      for (int k = 0; k < 3; ++k) Fv[i][k] = -bs[k] * V[i];
+  }
+  if (a.beta_field) {
+    shift_field_vflux<double, dim>(gm, V, sb, sB, Fv);
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+      for (int k = 0; k < 3; ++k) Fv[i][k] *= fs;
+  }
   bool bad = false;
 #pragma unroll
   for (int F = 0; F < kNF; ++F) {
+    const double base = (REP == kDEV ? r[F] - flat_value(F) : r[F]) - a.half_dt * Sr[F];
 #pragma unroll
     for (int l = 0; l < Q; ++l) {
-      double cf = 0;
-      if (has_flux(F)) {
+      double v = REP == kDEV ? base : L::w(l) * base;
+      if (has_flux(F) || (is_v(F) && a.shift_on)) {
 #pragma unroll
-        for (int k = 0; k < dim; ++k) cf += L::c(l, k) * Fl[F - kK][k];
+        for (int k = 0; k < dim; ++k) {
+          const double b = (REP == kDEV ? 1.0 : L::w(l) / kWb) *
+                           (has_flux(F) ? Fl[has_flux(F) ? F - kK : 0][k] : Fv[is_v(F) ? F - kV : 0][k]);
+          if (L::c(l, k) > 0) v += b;
+          if (L::c(l, k) < 0) v -= b;
+        }
       }
-      if (is_v(F) && a.beta_field) {
-#pragma unroll
-        for (int k = 0; k < dim; ++k) cf += L::c(l, k) * Fv[F - kV][k];
-      } else if (is_v(F) && a.shift_on) {
-#pragma unroll
-        for (int k = 0; k < dim; ++k) cf += L::c(l, k) * (-sb[k] * r[F]);
-      }
-      // f = w (rho + 3 c.F) - (dt/2) w S
-      double v;
-      if (REP == kDEV)
-        v = (r[F] - flat_value(F)) + 3.0 * cf - a.half_dt * Sr[F];
-      else
-        v = L::w(l) * (r[F] + 3.0 * cf) - a.half_dt * L::w(l) * Sr[F];
       bad |= !isfinite(v);
       Codec<S>::store(a.f + fidx<Q, S>((uint32_t)c, F, l), (decltype(Codec<S>::load(a.f)))v);
     }
@@ -1142,20 +1162,27 @@ __global__ void __launch_bounds__(256) k_sum64(const S* __restrict__ f, double* 
   }
 }
 
-// rho = rho~ + dt S(rho~)/2 in place (FP64), derivatives from aux64.
+// rho = rho~ + dt S(rho~)/2 (FP64), derivatives from aux64, into out: macro
+// itself, or a page-locked host array, whose writes then pass under the FP64
+// arithmetic that bounds this kernel.
 template <int Q>
-__global__ void __launch_bounds__(128) k_correct64(double* __restrict__ macro,
+__global__ void __launch_bounds__(128) k_correct64(const double* macro, double* out,
                                                    const double* __restrict__ aux64, Grid G,
                                                    double inv2dx, double inv4dx, double half_dt,
                                                    int slicing, int sources_on, double fluidP,
                                                    double bx, double by, double bz,
                                                    const double* __restrict__ beta_field) {
   const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= G.cells || !sources_on) return;
+  if (c >= G.cells || (!sources_on && out == macro)) return;
   const Nbr n = make_nbr(G, c);
   double r[kNF];
 #pragma unroll
   for (int F = 0; F < kNF; ++F) r[F] = macro[(int64_t)F * G.cells + c];
+  if (!sources_on) {
+#pragma unroll
+    for (int F = 0; F < kNF; ++F) out[(int64_t)F * G.cells + c] = r[F];
+    return;
+  }
   double A[3], D[3][6];
   derivatives<Q, double>(n, G.cells, aux64, inv2dx, inv4dx, A, D);
   double alpha, gm[6], K[6], V[3];
@@ -1171,7 +1198,7 @@ __global__ void __launch_bounds__(128) k_correct64(double* __restrict__ macro,
   }
   if (beta_field || bx != 0.0 || by != 0.0 || bz != 0.0) shift_sources<double>(sb, alpha, A, D, S);
 #pragma unroll
-  for (int F = 0; F < kNF; ++F) macro[(int64_t)F * G.cells + c] = r[F] + half_dt * S[F];
+  for (int F = 0; F < kNF; ++F) out[(int64_t)F * G.cells + c] = r[F] + half_dt * S[F];
 }
 
 // Christoffel symbols Gamma^k_ij (and the inverse metric, D) at a cell from
