@@ -46,6 +46,17 @@
 namespace lbnr {
 namespace {
 
+// What a cell costs besides its Q velocities, in velocities, in the plan's
+// run costs: the sources and fluxes. Without it 1D runs got too few blocks and
+// finished last (32 uneven runs, 256 x 1: 68.6 ms at 0, 67.9 at 4, 58.9 at 8, 58.6 at 20).
+constexpr double kCellCost = 8;
+// Between these many cells in all runs, blocks of 256 are sized for two per SM
+// where the caller leaves the number open: fewer, and a step waits for one
+// block's chain of passes, which more registers shorten; more, and the runs
+// miss the L2. ms, one against two per SM (SYNC): 31e3 cells 4.20 / 5.50, 230e3
+// 33.4 / 30.1, 1.7e6 125.5 / 113.0, 6.7e6 844 / 774, 18e6 2029 / 2396.
+constexpr int64_t kFewCells = 120000, kManyCells = 10000000;
+
 struct BatchRun {
   void* f[2];
   void* aux;
@@ -105,7 +116,7 @@ __device__ bool team_sync(const BatchParams& p, const Assign& A, int k) {
         atomicOr(p.flag, 2);
         break;
       }
-      __nanosleep(256);
+      __nanosleep(64);
     }
     __threadfence();
   }
@@ -194,7 +205,8 @@ __device__ void run_steps(const BatchParams& p, const BatchRun& R, const Assign&
 
 // Launch bounds: form 0 takes blocks of 256 threads with up to 255
 // registers a thread (one block per SM), form 1 blocks of 128 with up to 168
-// (three per SM), form 2 blocks of 128 with up to 128 (four per SM).
+// (three per SM), form 2 blocks of 128 with up to 128 (four per SM), form 3
+// blocks of 256 with up to 128 (two per SM).
 template <int FORM>
 struct BatchForm;
 template <>
@@ -208,6 +220,11 @@ struct BatchForm<1> {
 template <>
 struct BatchForm<2> {
   static constexpr int kThreads = 128, kMinBlocks = 4;
+};
+
+template <>
+struct BatchForm<3> {
+  static constexpr int kThreads = 256, kMinBlocks = 2;
 };
 
 template <class S, int REP, int FORM, bool LAG>
@@ -244,9 +261,9 @@ void* batch_kernel_form(int storage) {
 }
 
 // Form for a block size and a requested number of blocks per SM (0: the
-// form's own maximum).
-int form_for(int block, int per_sm) {
-  if (block == 256) return 0;
+// form's own maximum, chosen by the cells of all runs).
+int form_for(int block, int per_sm, int64_t cells) {
+  if (block == 256) return per_sm == 1 || (per_sm == 0 && (cells < kFewCells || cells > kManyCells)) ? 0 : 3;
   return per_sm == 4 ? 2 : 1;
 }
 
@@ -254,7 +271,8 @@ template <bool LAG>
 void* batch_kernel_mode(int storage, int form) {
   return form == 0 ? batch_kernel_form<0, LAG>(storage)
                    : form == 1 ? batch_kernel_form<1, LAG>(storage)
-                               : batch_kernel_form<2, LAG>(storage);
+                   : form == 2 ? batch_kernel_form<2, LAG>(storage)
+                               : batch_kernel_form<3, LAG>(storage);
 }
 
 void* batch_kernel(int storage, int form, int deriv_mode) {
@@ -329,7 +347,7 @@ void make_plan(lbnr_batch* b, int workers, const std::vector<char>& live) {
     const lbnr_run_desc& d = b->runs[r];
     const bool on = live.empty() || live[r];
     cost[r] = on ? (double)(d.grid.nx * d.grid.ny * d.grid.nz) *
-                       (double)std::max<int64_t>(d.steps, 1) * qv(d.vset)
+                       (double)std::max<int64_t>(d.steps, 1) * (qv(d.vset) + kCellCost)
                  : 0.0;
     total += cost[r];
   }
@@ -400,7 +418,9 @@ int live_runs(lbnr_batch* b, std::vector<char>& live) {
 int configure(lbnr_batch* b, int block, int ctas_per_sm) {
   if (block != 128 && block != 256) return bfail(b, LBNR_EINVAL, "block must be 128 or 256");
   if (ctas_per_sm < 0 || ctas_per_sm > 4) return bfail(b, LBNR_EINVAL, "ctas_per_sm must be 0..4");
-  const int form = form_for(block, ctas_per_sm);
+  int64_t cells = 0;
+  for (const lbnr_run_desc& d : b->runs) cells += d.grid.nx * d.grid.ny;
+  const int form = form_for(block, ctas_per_sm, cells);
   void* kern = batch_kernel(b->opts.storage, form, b->opts.deriv_mode);
   // the kernel uses no shared memory to speak of: give the SM's unified
   // cache to L1
