@@ -48,22 +48,27 @@ struct Args {
   int slicing;
 };
 
-// Distribution layout: the tile-blocked words of the 16-field scheme, with
-// the 37 fields padded to whole words. A word holds kV consecutive fields of
-// one cell and velocity (four for FP32: 10 words per velocity, slots 37-39
-// held at zero; one for FP64: 37 words). The values of the 32 cells of a tile
-// form one contiguous block, ordered by velocity, then word, then cell.
+// Distribution layout: the tile-blocked words of the 16-field scheme. A word
+// holds kV consecutive fields of one cell and velocity (FP32: nine words of four
+// and the last field by itself; FP64: 37 words of one). The values of the 32
+// cells of a tile form one contiguous block, ordered by velocity, then word,
+// then cell. (Padded to ten words, FP32 moved 6080 bytes a cell-step instead of
+// 5624: 869 against 819 us a step at 96^3, 2057 against 1940 at 128^3.)
 template <class S>
-constexpr int kWords = (kNFA + Codec<S>::kV - 1) / Codec<S>::kV;
+constexpr int kWords = kNFA / Codec<S>::kV;
 template <class S>
-constexpr int kSlots = kWords<S> * Codec<S>::kV;
+constexpr int kTail = kNFA % Codec<S>::kV;  // fields past the last whole word
+template <class S>
+constexpr bool kTailed = kTail<S> > 0;
 
 template <int Q, class S>
 __host__ __device__ __forceinline__ size_t ad_fidx(uint32_t c, int F, int l) {
   constexpr int V = Codec<S>::kV;
   constexpr int NW = kWords<S>;
-  return (((size_t)(c >> 5) * (size_t)(NW * Q) + (size_t)(l * NW + F / V)) * lbnr::kTileCells +
-          (c & 31u)) * V + (size_t)(F % V);
+  static_assert(kTail<S> <= 1, "one field past the words");
+  const size_t row = ((size_t)(c >> 5) * Q + l) * (size_t)(kNFA * lbnr::kTileCells);
+  return F < NW * V ? row + ((size_t)(F / V) * lbnr::kTileCells + (c & 31u)) * V + (size_t)(F % V)
+                    : row + (size_t)(NW * V) * lbnr::kTileCells + (c & 31u);
 }
 
 // Whole words: read-only path, streaming (last use) load, streaming store.
@@ -113,17 +118,18 @@ __device__ __forceinline__ void ad_field_terms(int F, const C rt[kNFA], const C 
       if (kk == k) b[kk] = three_omega * fk;
   }
 }
-// The same for a word's slot F: zero for the padding slots (F >= 37).
-template <int dim, class S, class C>
-__device__ __forceinline__ void ad_word_terms(int F, const C rt[kNFA], const C rho[kNF],
-                                              const C Sr[kNF], const C Fl[6][3], C aQ,
-                                              const C aK[6], const Args<S, C>& a, C& cf, C b[3]) {
-  if (F < kNFA) {
-    ad_field_terms<dim, C>(F, rt, rho, Sr, Fl, aQ, aK, a.omega, a.sigma, cf, b);
-  } else {
-    cf = C(0);
-    b[0] = b[1] = b[2] = C(0);
+
+// One value of velocity l relaxed with its field's coefficient and fluxes.
+template <int Q, class C>
+__device__ __forceinline__ C relax_value(C v, int l, C omc, C cf, const C b[3]) {
+  using L = Lattice<Q>;
+  C t = cf;
+#pragma unroll
+  for (int k = 0; k < L::kDim; ++k) {
+    if (L::c(l, k) > 0) t += b[k];
+    if (L::c(l, k) < 0) t -= b[k];
   }
+  return fma(omc, v, C(L::w(l)) * t);
 }
 
 // One step: moments, sources (A and D from the cell's own moments), the
@@ -152,9 +158,12 @@ __global__ void __launch_bounds__(128, MINB) k_ad_collide(const Args<S, C> a) {
       C v[V];
       unpack_word<S>(ld_word_keep<S>(a.fin + ad_fidx<Q, S>(n.c, V * m, l)), v);
 #pragma unroll
-      for (int i = 0; i < V; ++i)
-        if (V * m + i < kNFA) rt[V * m + i] += v[i];
+      for (int i = 0; i < V; ++i) rt[V * m + i] += v[i];
     }
+  }
+  if (kTailed<S>) {
+#pragma unroll
+    for (int l = 0; l < Q; ++l) rt[kNFA - 1] += Codec<S>::load_keep(a.fin + ad_fidx<Q, S>(n.c, kNFA - 1, l));
   }
   // reported after the update pass, so that no global write stands between
   // the two passes' loads
@@ -196,7 +205,7 @@ __global__ void __launch_bounds__(128, MINB) k_ad_collide(const Args<S, C> a) {
     for (int l = 0; l < Q; ++l) vw[l] = ld_word_last<S>(a.fin + ad_fidx<Q, S>(n.c, V * m, l));
     C cf[V], b[V][3];
 #pragma unroll
-    for (int i = 0; i < V; ++i) ad_word_terms<dim>(V * m + i, rt, rho, Sr, Fl, aQ, aK, a, cf[i], b[i]);
+    for (int i = 0; i < V; ++i) ad_field_terms<dim, C>(V * m + i, rt, rho, Sr, Fl, aQ, aK, a.omega, a.sigma, cf[i], b[i]);
 #pragma unroll
     for (int l = 0; l < Q; ++l) {
       C v[V], out[V];
@@ -209,10 +218,19 @@ __global__ void __launch_bounds__(128, MINB) k_ad_collide(const Args<S, C> a) {
           if (L::c(l, k) > 0) t += b[i][k];
           if (L::c(l, k) < 0) t -= b[i][k];
         }
-        // padding slots stay zero
-        out[i] = V * m + i < kNFA ? fma(a.omc, v[i], C(L::w(l)) * t) : C(0);
+        out[i] = fma(a.omc, v[i], C(L::w(l)) * t);
       }
       store_word<S>(a.fout + ad_fidx<Q, S>(n.at(L::c(l, 0), L::c(l, 1), L::c(l, 2)), V * m, l), out);
+    }
+  }
+  if constexpr (kTailed<S>) {
+    C cf, b[3];
+    ad_field_terms<dim, C>(kNFA - 1, rt, rho, Sr, Fl, aQ, aK, a.omega, a.sigma, cf, b);
+#pragma unroll
+    for (int l = 0; l < Q; ++l) {
+      const C v = Codec<S>::load(a.fin + ad_fidx<Q, S>(n.c, kNFA - 1, l));
+      Codec<S>::store(a.fout + ad_fidx<Q, S>(n.at(L::c(l, 0), L::c(l, 1), L::c(l, 2)), kNFA - 1, l),
+                      relax_value<Q, C>(v, l, a.omc, cf, b));
     }
   }
   if (bad) atomicOr(a.flag, 1);
@@ -289,11 +307,6 @@ __global__ void __launch_bounds__(128) k_ad_init(const double* __restrict__ fiel
       Codec<S>::store(f + ad_fidx<Q, S>((uint32_t)c, F, l), (decltype(Codec<S>::load(f)))val);
     }
   }
-  // padding slots of the last word
-#pragma unroll
-  for (int F = kNFA; F < kSlots<S>; ++F)
-#pragma unroll
-    for (int l = 0; l < Q; ++l) Codec<S>::store(f + ad_fidx<Q, S>((uint32_t)c, F, l), 0.0f);
   if (bad) atomicOr(flag, 1);
 }
 
@@ -347,7 +360,7 @@ constexpr int kTileCells = 32;
 
 template <class S>
 __host__ __device__ constexpr uint32_t tma_stage(int Q) {
-  return (uint32_t)(kSlots<S> * Q * kTileCells * sizeof(S));
+  return (uint32_t)(kNFA * Q * kTileCells * sizeof(S));
 }
 // Stages that fit the 227 KB of shared memory (at most 4).
 template <class S>
@@ -405,7 +418,7 @@ __global__ void __launch_bounds__(32 * (NS * P + 1), 1)
         const uint32_t fb = smem_u32(&bars[s]);
         mbar_expect_tx(fb, STAGEB);
         bulk_load(smem_u32(stages + (size_t)s * STAGEB),
-                  a.fin + (size_t)tile * (size_t)(kSlots<S> * Q * T), STAGEB, fb);
+                  a.fin + (size_t)tile * (size_t)(kNFA * Q * T), STAGEB, fb);
         issued = j + 1;
       }
       // leave only when every copy started here has landed
@@ -456,7 +469,7 @@ __global__ void __launch_bounds__(32 * (NS * P + 1), 1)
         }
 #pragma unroll
         for (int i = 0; i < V; ++i)
-          if (V * w + i < kNFA) rt[V * w + i] = sum[i];
+          rt[V * w + i] = sum[i];
       }
     } else {
       // words 2jj (lanes g = 0) and 2jj + 1 (g = 1), swapped between partner
@@ -476,8 +489,8 @@ __global__ void __launch_bounds__(32 * (NS * P + 1), 1)
 #pragma unroll
         for (int i = 0; i < V; ++i) {
           const C other = __shfl_xor_sync(0xffffffffu, sum[i], 16);
-          if (V * (2 * jj) + i < kNFA) rt[V * (2 * jj) + i] = g ? other : sum[i];
-          if (V * (2 * jj + 1) + i < kNFA) rt[V * (2 * jj + 1) + i] = g ? sum[i] : other;
+          rt[V * (2 * jj) + i] = g ? other : sum[i];
+          rt[V * (2 * jj + 1) + i] = g ? sum[i] : other;
         }
       }
       if constexpr (NW % 2 == 1) {
@@ -493,8 +506,14 @@ __global__ void __launch_bounds__(32 * (NS * P + 1), 1)
         }
 #pragma unroll
         for (int i = 0; i < V; ++i)
-          if (V * (NW - 1) + i < kNFA) rt[V * (NW - 1) + i] = sum[i];
+          rt[V * (NW - 1) + i] = sum[i];
       }
+    }
+    if constexpr (kTailed<S>) {  // both lanes of a pair
+      C t = C(0);
+#pragma unroll
+      for (int l = 0; l < Q; ++l) t += C(st[ad_fidx<Q, S>((uint32_t)ci, kNFA - 1, l)]);
+      rt[kNFA - 1] = t;
     }
     bool bad;
     {
@@ -552,7 +571,7 @@ __global__ void __launch_bounds__(32 * (NS * P + 1), 1)
       for (int w = 0; w < NW; ++w) {
         C cf[V], b[V][3];
 #pragma unroll
-        for (int i = 0; i < V; ++i) ad_word_terms<dim>(V * w + i, rt, rho, Sr, Fl, aQ, aK, a, cf[i], b[i]);
+        for (int i = 0; i < V; ++i) ad_field_terms<dim, C>(V * w + i, rt, rho, Sr, Fl, aQ, aK, a.omega, a.sigma, cf[i], b[i]);
         relax(w, cf, b, valid);
       }
     } else {
@@ -561,8 +580,8 @@ __global__ void __launch_bounds__(32 * (NS * P + 1), 1)
         C cf0[V], b0[V][3], cf1[V], b1[V][3], cf[V], b[V][3];
 #pragma unroll
         for (int i = 0; i < V; ++i) {
-          ad_word_terms<dim>(V * (2 * jj) + i, rt, rho, Sr, Fl, aQ, aK, a, cf0[i], b0[i]);
-          ad_word_terms<dim>(V * (2 * jj + 1) + i, rt, rho, Sr, Fl, aQ, aK, a, cf1[i], b1[i]);
+          ad_field_terms<dim, C>(V * (2 * jj) + i, rt, rho, Sr, Fl, aQ, aK, a.omega, a.sigma, cf0[i], b0[i]);
+          ad_field_terms<dim, C>(V * (2 * jj + 1) + i, rt, rho, Sr, Fl, aQ, aK, a.omega, a.sigma, cf1[i], b1[i]);
           cf[i] = g ? cf1[i] : cf0[i];
 #pragma unroll
           for (int k = 0; k < 3; ++k) b[i][k] = g ? b1[i][k] : b0[i][k];
@@ -572,9 +591,19 @@ __global__ void __launch_bounds__(32 * (NS * P + 1), 1)
       if constexpr (NW % 2 == 1) {
         C cf[V], b[V][3];
 #pragma unroll
-        for (int i = 0; i < V; ++i) ad_word_terms<dim>(V * (NW - 1) + i, rt, rho, Sr, Fl, aQ, aK, a, cf[i], b[i]);
+        for (int i = 0; i < V; ++i) ad_field_terms<dim, C>(V * (NW - 1) + i, rt, rho, Sr, Fl, aQ, aK, a.omega, a.sigma, cf[i], b[i]);
         relax(NW - 1, cf, b, valid && g == 0);
       }
+    }
+    if constexpr (kTailed<S>) {
+      C cf, b[3];
+      ad_field_terms<dim, C>(kNFA - 1, rt, rho, Sr, Fl, aQ, aK, a.omega, a.sigma, cf, b);
+#pragma unroll
+      for (int l = 0; l < Q; ++l)
+        Codec<S>::store_if(
+            a.fout + ad_fidx<Q, S>(n.at(L::c(l, 0), L::c(l, 1), L::c(l, 2)), kNFA - 1, l),
+            relax_value<Q, C>(C(st[ad_fidx<Q, S>((uint32_t)ci, kNFA - 1, l)]), l, a.omc, cf, b),
+            valid && g == P - 1);
     }
     if (bad) atomicOr(a.flag, 1);
     __syncwarp();
