@@ -146,8 +146,8 @@ struct Impl {
   // One launch form: both passes in one launch (k_step), or one pass a launch.
   // Then FP64, bound by its operations, takes the sums of the moment pass
   // again (64^3: 867 us a step, 914 without); the other storages read every
-  // word in pass 1, which brings them on chip for pass 2 (256^3 FP16: 4.29 ms
-  // a step, 4.41 with the sums).
+  // word in pass 1, which brings them on chip for pass 2 (256^3 FP16: 4.18 ms
+  // a step; about 0.1 more with the sums).
   template <int LAYOUT, int SHIFT, bool H, int TPB, int MINB, int LAGMINB>
   static cudaError_t launch_form(const LaunchCtx& L, const StepArgs<S, C>& a, bool one_launch) {
     const unsigned grid = grid_for(L.cells, TPB);
@@ -306,7 +306,7 @@ struct Impl {
     const unsigned grid = grid_for(L.cells, 256);
     const S* fp = static_cast<const S*>(f);
     C* ap = static_cast<C*>(L.aux);
-    C* sp = static_cast<C*>(L.sums);
+    C* sp = sizeof(C) == 8 ? static_cast<C*>(L.sums) : nullptr;  // as launch_form takes them
     if (layout == kPingPong) k_aux<Q, S, C, REP, kPingPong><<<grid, 256, 0, L.st>>>(fp, ap, sp, G);
     else if (layout == kAAEven) k_aux<Q, S, C, REP, kAAEven><<<grid, 256, 0, L.st>>>(fp, ap, sp, G);
     else k_aux<Q, S, C, REP, kAAOdd><<<grid, 256, 0, L.st>>>(fp, ap, sp, G);

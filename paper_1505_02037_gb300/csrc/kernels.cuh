@@ -314,7 +314,6 @@ struct StepArgs {
   const S* fin;
   S* fout;
   const C* aux;  // 7 planes: ln(alpha~) or log1p(alpha~ - 1); gamma~ or gamma~ - delta
-  const C* sums; // SYNC: 2 planes the moment pass writes beside them (aux_body)
   // Reading R17 (LAG): aux holds the previous step's corrected lapse and
   // metric in that form, and the step writes its own corrected ones to
   // aux_out for the next step. nullptr: aux holds this step's rho~ (R5).
@@ -335,6 +334,10 @@ struct StepArgs {
   // it, whose central differences give B_k^i.
   C beta[3];
   const double* beta_field;
+  // SYNC: 2 planes the moment pass writes beside aux (aux_body). Last on
+  // purpose: with it after aux the compiler schedules the loads of the other
+  // arguments so that the LAG collide at 256^3 FP32 takes 6.76 instead of 6.28 ms.
+  const C* sums;
 };
 
 // Reading R17: the corrected lapse and metric of this step, in the stencil
@@ -519,12 +522,12 @@ __device__ __forceinline__ typename Codec<S>::W load_word(const S* p) {
   else
     return POL == kKeep ? WordIO<S>::ldw_keep(p) : POL == kLast ? WordIO<S>::ldw(p) : WordIO<S>::ldw_coh(p);
 }
-// The four FP32 values of a word as two pairs. Sums, relaxation and fluxes run
-// on pairs (one instruction for two values, each rounded as by the scalar
-// instruction): 16-bit storage is bound by issue slots, and the other forms
-// wait less between their loads.
+// The four FP32 values of a word as two pairs. The sums run on pairs (one
+// instruction for two values, each rounded as by the scalar instruction):
+// 16-bit storage waits on its instructions (256^3 FP16 collide 3.53 to 3.37 ms).
+// The relaxation gains nothing from pairs (3.49 ms): they want neighbouring
+// registers, which costs the compiler freedom between pass 2's loads.
 __device__ __forceinline__ float2 pair(float a) { return make_float2(a, a); }
-__device__ __forceinline__ float2 neg(float2 a) { return make_float2(-a.x, -a.y); }
 template <class S>
 __device__ __forceinline__ void unpack_pairs(typename Codec<S>::W w, float2 v[2]) {
   float t[4];
@@ -586,7 +589,7 @@ __device__ __forceinline__ void word_sums(const S* __restrict__ f, const Nbr& n,
 // aux: ln(alpha~) and gamma~ (or their deviations) for the stencil; sums:
 // alpha~ itself and (words of four fields) the other field of the second word,
 // K_xx. With them the collide pass needs no sums of the words that this pass
-// has summed already.
+// has summed already; nullptr where it takes its own.
 template <class S>
 constexpr int kAuxWords = Codec<S>::kV == 1 ? 7 : 2;  // words holding fields 0..6
 template <int Q, class S, class C, int REP, int LAYOUT, int POL>
@@ -597,8 +600,10 @@ __device__ __forceinline__ void aux_body(const S* __restrict__ f, C* __restrict_
 #pragma unroll
   for (int m = 0; m < kAuxWords<S>; ++m) word_sums<Q, S, C, REP, LAYOUT, POL>(f, n, m, s + V * m);
   if (!valid) return;
-  sums[n.c] = s[0];
-  if (V > 1) sums[cells + n.c] = s[V > 1 ? 7 : 0];
+  if (sums) {
+    sums[n.c] = s[0];
+    if (V > 1) sums[cells + n.c] = s[V > 1 ? 7 : 0];
+  }
   C* p = aux + n.c;
   p[0] = REP == kDEV ? log1p(s[0]) : log(s[0]);
 #pragma unroll
@@ -749,7 +754,7 @@ __device__ __forceinline__ bool collide_body(const StepArgs<S, C>& a, const Nbr&
         else
           Codec<S>::store_if(dst, out, valid);
       }
-    } else if constexpr (!kLean) {
+    } else {
       C b[V][3];
 #pragma unroll
       for (int i = 0; i < V; ++i)
@@ -771,39 +776,6 @@ __device__ __forceinline__ bool collide_body(const StepArgs<S, C>& a, const Nbr&
           }
           out[i] = REP == kDEV ? fma(a.omc, v[i], t) : fma(a.omc, v[i], C(L::w(l)) * t);
         }
-        S* dst = a.fout + write_index<Q, LAYOUT, S>(n, V * m, l);
-        if (LAYOUT == kPingPong)
-          WordIO<S>::stw(dst, Codec<S>::pack(out));
-        else
-          WordIO<S>::stw_if(dst, Codec<S>::pack(out), valid);
-      }
-    } else {
-      float2 c2[2], b[2][3];
-#pragma unroll
-      for (int p = 0; p < 2; ++p) {
-        const int F = V * m + 2 * p;
-        c2[p] = make_float2(cf[F], cf[F + 1]);
-#pragma unroll
-        for (int k = 0; k < 3; ++k) b[p][k] = make_float2(flux(F, k), flux(F + 1, k));
-      }
-#pragma unroll
-      for (int l = 0; l < Q; ++l) {
-        float2 v[2];
-        unpack_pairs<S>(vw[l], v);
-#pragma unroll
-        for (int p = 0; p < 2; ++p) {
-          float2 t = c2[p];
-          if (fluxed(V * m + 2 * p) || fluxed(V * m + 2 * p + 1)) {
-#pragma unroll
-            for (int k = 0; k < dim; ++k) {
-              if (L::c(l, k) > 0) t = __fadd2_rn(t, b[p][k]);
-              if (L::c(l, k) < 0) t = __fadd2_rn(t, neg(b[p][k]));
-            }
-          }
-          v[p] = __ffma2_rn(pair(a.omc), v[p],
-                            REP == kDEV ? t : __fmul2_rn(pair((float)L::w(l)), t));
-        }
-        const float out[4] = {v[0].x, v[0].y, v[1].x, v[1].y};
         S* dst = a.fout + write_index<Q, LAYOUT, S>(n, V * m, l);
         if (LAYOUT == kPingPong)
           WordIO<S>::stw(dst, Codec<S>::pack(out));
@@ -870,7 +842,7 @@ __global__ void __launch_bounds__(256) k_aux(const S* __restrict__ f, C* __restr
 // late (7107: the passes move apart), an L2 prefetch a unit ahead (6913), the
 // words of pass 1 staged in shared memory (7557), 10 or 12 warps per SM (7608:
 // the words no longer stay in the L2). 16-bit storage gains nothing (4261
-// against 4290: it waits on its conversions, not on HBM), and D2Q9 loses (240
+// against 4176: it waits on its conversions, not on HBM), and D2Q9 loses (240
 // against 227), so both keep two launches; so does FP64, bound by its operations.
 __device__ __forceinline__ unsigned ld_acquire(const unsigned* p) {
   unsigned v;
