@@ -522,11 +522,12 @@ __device__ __forceinline__ typename Codec<S>::W load_word(const S* p) {
   else
     return POL == kKeep ? WordIO<S>::ldw_keep(p) : POL == kLast ? WordIO<S>::ldw(p) : WordIO<S>::ldw_coh(p);
 }
-// The four FP32 values of a word as two pairs. The sums run on pairs (one
-// instruction for two values, each rounded as by the scalar instruction):
-// 16-bit storage waits on its instructions (256^3 FP16 collide 3.53 to 3.37 ms).
-// The relaxation gains nothing from pairs (3.49 ms): they want neighbouring
-// registers, which costs the compiler freedom between pass 2's loads.
+// The four FP32 values of a word as two pairs: one instruction for two values,
+// each rounded as by the scalar instruction. The 3D forms sum on pairs (256^3
+// FP16 collide 3.53 to 3.37 ms). The relaxation uses them with 4-byte storage
+// only (149 x 101 x 67 FP32 deviations in place, a pass of 100 steps: 50.4 ms,
+// 52.7 with scalars); with 16 bits the neighbouring registers they want cost the
+// compiler freedom between pass 2's loads (3.49 ms instead of 3.37).
 __device__ __forceinline__ float2 pair(float a) { return make_float2(a, a); }
 template <class S>
 __device__ __forceinline__ void unpack_pairs(typename Codec<S>::W w, float2 v[2]) {
@@ -753,6 +754,39 @@ __device__ __forceinline__ bool collide_body(const StepArgs<S, C>& a, const Nbr&
           Codec<S>::store(dst, out);
         else
           Codec<S>::store_if(dst, out, valid);
+      }
+    } else if constexpr (kLean && sizeof(S) == 4) {
+      float2 c2[2], b[2][3];
+#pragma unroll
+      for (int p = 0; p < 2; ++p) {
+        const int F = V * m + 2 * p;
+        c2[p] = make_float2(cf[F], cf[F + 1]);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) b[p][k] = make_float2(flux(F, k), flux(F + 1, k));
+      }
+#pragma unroll
+      for (int l = 0; l < Q; ++l) {
+        float2 v[2];
+        unpack_pairs<S>(vw[l], v);
+#pragma unroll
+        for (int p = 0; p < 2; ++p) {
+          float2 t = c2[p];
+          if (fluxed(V * m + 2 * p) || fluxed(V * m + 2 * p + 1)) {
+#pragma unroll
+            for (int k = 0; k < dim; ++k) {
+              if (L::c(l, k) > 0) t = __fadd2_rn(t, b[p][k]);
+              if (L::c(l, k) < 0) t = __fadd2_rn(t, make_float2(-b[p][k].x, -b[p][k].y));
+            }
+          }
+          v[p] = __ffma2_rn(pair(a.omc), v[p],
+                            REP == kDEV ? t : __fmul2_rn(pair((float)L::w(l)), t));
+        }
+        const float out[4] = {v[0].x, v[0].y, v[1].x, v[1].y};
+        S* dst = a.fout + write_index<Q, LAYOUT, S>(n, V * m, l);
+        if (LAYOUT == kPingPong)
+          WordIO<S>::stw(dst, Codec<S>::pack(out));
+        else
+          WordIO<S>::stw_if(dst, Codec<S>::pack(out), valid);
       }
     } else {
       C b[V][3];
