@@ -180,8 +180,8 @@ __device__ void run_steps(const BatchParams& p, const BatchRun& R, const Assign&
       for (int64_t base = A.rank * B; base < cells; base += (int64_t)A.team * B) {
         const int64_t c = base + threadIdx.x;
         if (c < cells)
-          aux_body<Q, S, C, REP, kPingPong, kCoherent>(
-              a.fin, aux, kReuse<C> ? aux + 7 * cells : nullptr, cells, make_nbr(a.G, c), true);
+          aux_body<Q, S, C, REP, kPingPong, kCoherent, kReuse<C>>(
+              a.fin, aux, aux + 7 * cells, cells, make_nbr(a.G, c), true);
       }
       if (!team_sync(p, A, k++)) return;
     }

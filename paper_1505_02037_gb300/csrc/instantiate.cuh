@@ -306,10 +306,11 @@ struct Impl {
     const unsigned grid = grid_for(L.cells, 256);
     const S* fp = static_cast<const S*>(f);
     C* ap = static_cast<C*>(L.aux);
-    C* sp = sizeof(C) == 8 ? static_cast<C*>(L.sums) : nullptr;  // as launch_form takes them
-    if (layout == kPingPong) k_aux<Q, S, C, REP, kPingPong><<<grid, 256, 0, L.st>>>(fp, ap, sp, G);
-    else if (layout == kAAEven) k_aux<Q, S, C, REP, kAAEven><<<grid, 256, 0, L.st>>>(fp, ap, sp, G);
-    else k_aux<Q, S, C, REP, kAAOdd><<<grid, 256, 0, L.st>>>(fp, ap, sp, G);
+    C* sp = static_cast<C*>(L.sums);
+    constexpr bool kSums = sizeof(C) == 8;  // as launch_form takes them
+    if (layout == kPingPong) k_aux<Q, S, C, REP, kPingPong, kSums><<<grid, 256, 0, L.st>>>(fp, ap, sp, G);
+    else if (layout == kAAEven) k_aux<Q, S, C, REP, kAAEven, kSums><<<grid, 256, 0, L.st>>>(fp, ap, sp, G);
+    else k_aux<Q, S, C, REP, kAAOdd, kSums><<<grid, 256, 0, L.st>>>(fp, ap, sp, G);
     return cudaGetLastError();
   }
 

@@ -589,11 +589,13 @@ __device__ __forceinline__ void word_sums(const S* __restrict__ f, const Nbr& n,
 // ---------------------------------------------------------------------------
 // aux: ln(alpha~) and gamma~ (or their deviations) for the stencil; sums:
 // alpha~ itself and (words of four fields) the other field of the second word,
-// K_xx. With them the collide pass needs no sums of the words that this pass
-// has summed already; nullptr where it takes its own.
+// K_xx. With them (SUMS) the collide pass needs no sums of the words that this
+// pass has summed already. Compiled in: as a question asked at run time they
+// cost k_aux of 16-bit storage 5 registers and a quarter of its warps (1000^2
+// D2Q9 FP16: a step 144.4 us, 142.0 without).
 template <class S>
 constexpr int kAuxWords = Codec<S>::kV == 1 ? 7 : 2;  // words holding fields 0..6
-template <int Q, class S, class C, int REP, int LAYOUT, int POL>
+template <int Q, class S, class C, int REP, int LAYOUT, int POL, bool SUMS>
 __device__ __forceinline__ void aux_body(const S* __restrict__ f, C* __restrict__ aux, C* sums,
                                          int64_t cells, const Nbr& n, bool valid) {
   constexpr int V = Codec<S>::kV;
@@ -601,9 +603,9 @@ __device__ __forceinline__ void aux_body(const S* __restrict__ f, C* __restrict_
 #pragma unroll
   for (int m = 0; m < kAuxWords<S>; ++m) word_sums<Q, S, C, REP, LAYOUT, POL>(f, n, m, s + V * m);
   if (!valid) return;
-  if (sums) {
+  if constexpr (SUMS) {
     sums[n.c] = s[0];
-    if (V > 1) sums[cells + n.c] = s[V > 1 ? 7 : 0];
+    if constexpr (V > 1) sums[cells + n.c] = s[7];
   }
   C* p = aux + n.c;
   p[0] = REP == kDEV ? log1p(s[0]) : log(s[0]);
@@ -836,12 +838,12 @@ __global__ void __launch_bounds__(TPB, HOLD ? 1 : MINB) k_collide(const StepArgs
     atomicOr(a.flag, 1);
 }
 
-template <int Q, class S, class C, int REP, int LAYOUT>
+template <int Q, class S, class C, int REP, int LAYOUT, bool SUMS>
 __global__ void __launch_bounds__(256) k_aux(const S* __restrict__ f, C* __restrict__ aux, C* sums,
                                              Grid G) {
   const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (c < G.cells)
-    aux_body<Q, S, C, REP, LAYOUT, kKeep>(f, aux, sums, G.cells, make_nbr(G, c), true);
+    aux_body<Q, S, C, REP, LAYOUT, kKeep, SUMS>(f, aux, sums, G.cells, make_nbr(G, c), true);
 }
 
 // ---------------------------------------------------------------------------
@@ -910,7 +912,7 @@ __global__ void __launch_bounds__(TPB, MINB) k_step(const StepArgs<S, C> a, C* a
       if (moment_tile(s, t, tile)) {
         const int64_t cell = (int64_t)tile * 32 + lane;
         const bool valid = cell < cells;
-        aux_body<Q, S, C, REP, LAYOUT, LAYOUT == kPingPong ? kKeep : kCoherent>(
+        aux_body<Q, S, C, REP, LAYOUT, LAYOUT == kPingPong ? kKeep : kCoherent, true>(
             a.fin, aux, sums, cells, make_nbr(a.G, valid ? cell : cells - 1), valid);
       }
       __syncwarp();
