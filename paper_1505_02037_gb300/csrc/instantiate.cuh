@@ -45,7 +45,8 @@ LBNR_VARIANTS(19, 8, 0, {0, 1, false, 0, 0, 0}, {1, 1, false, 2, 1, 32}, {2, 1, 
 // FP32 and 16-bit storage: one lane per cell, word by word. (Forms with two
 // lanes per cell split a word's fields between the lanes; on the word
 // layout they ran at half the speed and are not offered.) The re-read forms
-// come in three block shapes: 128 threads x 3 blocks per SM (168 registers),
+// come in three block shapes: 128 threads x 3 blocks per SM (168 registers; 2
+// blocks where launch_generic says so),
 // 64 x 4 and 128 x 2 (255 registers, 8 warps per SM: fewer cells resident,
 // so more of the update pass's re-read stays in L2). Form 0, what a context
 // runs until another one is chosen, is for D3Q19 the one that is fastest over
@@ -143,53 +144,56 @@ struct Impl {
     return cudaGetLastError();
   }
 
-  // One launch form: both passes in one launch (k_step), or one pass a launch.
-  // Then FP64, bound by its operations, takes the sums of the moment pass
-  // again (64^3: 867 us a step, 914 without); the other storages read every
-  // word in pass 1, which brings them on chip for pass 2 (256^3 FP16: 4.18 ms
-  // a step; about 0.1 more with the sums).
-  template <int LAYOUT, int SHIFT, bool H, int TPB, int MINB, int LAGMINB>
-  static cudaError_t launch_form(const LaunchCtx& L, const StepArgs<S, C>& a, bool one_launch) {
-    const unsigned grid = grid_for(L.cells, TPB);
-    if constexpr (!H && kOneLaunch) {
-      if (one_launch && !a.aux_out) return launch_step<LAYOUT, SHIFT, TPB, MINB>(L, a);
-    }
-    if (a.aux_out)
-      k_collide<Q, S, C, REP, LAYOUT, H, SHIFT, true, false, TPB, LAGMINB><<<grid, TPB, 0, L.st>>>(a);
-    else
-      k_collide<Q, S, C, REP, LAYOUT, H, SHIFT, false, sizeof(C) == 8, TPB, MINB>
-          <<<grid, TPB, 0, L.st>>>(a);
+  // One pass a launch. FP64, bound by its operations, takes the sums of the
+  // moment pass again (64^3: 867 us a step, 914 without); the other storages
+  // read every word in pass 1, which brings them on chip for pass 2 (256^3 FP16:
+  // 4.18 ms a step; about 0.1 more with the sums).
+  template <int LAYOUT, int SHIFT, bool H, bool LAGW, int TPB, int MINB>
+  static cudaError_t launch_collide(const LaunchCtx& L, const StepArgs<S, C>& a) {
+    k_collide<Q, S, C, REP, LAYOUT, H, SHIFT, LAGW, sizeof(C) == 8 && !LAGW, TPB, MINB>
+        <<<grid_for(L.cells, TPB), TPB, 0, L.st>>>(a);
     return cudaGetLastError();
   }
 
+  // The default shape is 128 threads sized for 3 blocks per SM, and for 2 where
+  // 168 registers cost more than the third block gives: word by word at the odd
+  // AA step, which holds a field group's Q words and reads and writes at
+  // neighbours, and in D3Q19 FP32 storage under LAG (128^3, us a step: 772 with
+  // 2, 836 with 3). FP64 takes blocks of 64 sized for 6: bound by its operations,
+  // it waits for the SM with the most cells, and hides what its 168 registers
+  // spill (430 to 780 bytes); with the lagged-field writes sized for 4, which
+  // spills nothing.
   template <int LAYOUT, int VI>
   static cudaError_t launch_generic(const LaunchCtx& L, const StepArgs<S, C>& a, bool one_launch) {
     constexpr VariantSpec x = VT::v[VI];
     static_assert(x.P == 1, "one thread per cell");
-    // The default shape, 128 threads sized for 3 blocks per SM, takes 2 where
-    // it would spill: word by word at the odd AA step, which holds a field
-    // group's Q words and reads and writes at neighbours, and in FP64 with the
-    // lagged-field writes. FP64 takes the same in blocks of 64: bound by its
-    // operations, it waits for the SM with the most cells.
     constexpr bool kWords = Codec<S>::kV > 1;
     constexpr int TPB = x.tpb > 0 ? x.tpb : kWords ? 128 : 64;
     constexpr int MINB = x.minb > 0 ? x.minb : kWords ? (LAYOUT == kAAOdd ? 2 : 3) : 6;
-    constexpr int LAGMINB = kWords ? MINB : 4;
-    return launch_form<LAYOUT, 0, x.hold, TPB, MINB, LAGMINB>(L, a, one_launch);
+    constexpr int LAGMINB = !kWords ? 4 : kOneLaunch && x.minb == 0 ? 2 : MINB;
+    if (a.aux_out) return launch_collide<LAYOUT, 0, x.hold, true, TPB, LAGMINB>(L, a);
+    if constexpr (!x.hold && kOneLaunch) {
+      if (one_launch) return launch_step<LAYOUT, 0, TPB, MINB>(L, a);
+    }
+    return launch_collide<LAYOUT, 0, x.hold, false, TPB, MINB>(L, a);
   }
 
-  // Registers of the shift forms. FP64 (value by value): 3 blocks of 128
-  // threads per SM (the FP64 step is bound by its arithmetic; 8.9 against
-  // 9.3 ms at 128^3). FP32 and 16-bit storage (word by word): 3 blocks with
-  // a constant shift, which fits 168 registers without spills outside the
-  // odd AA step, else 2 (255 registers; 3 would spill).
+  // The shift forms. FP64 (value by value): 3 blocks of 128 threads per SM (bound
+  // by its arithmetic; 8.9 against 9.3 ms at 128^3). FP32 storage on D3Q19: 64 x 4,
+  // as without a shift, in one launch and under LAG (128^3, constant shift under
+  // LAG: 774 us, 841 at 128 x 3 whose 168 registers spill 88 bytes). The others
+  // word by word: 3 blocks of 128 with a constant shift, 2 with a shift field
+  // and at the odd AA step (255 registers).
   template <int LAYOUT, int SHIFT>
   static cudaError_t launch_shifted(const LaunchCtx& L, const StepArgs<S, C>& a) {
-    if constexpr (kOneLaunch) {
-      if (fused(L, 0)) return launch_step<LAYOUT, SHIFT, 64, 4>(L, a);
-    }
     constexpr int MINB = sizeof(C) == 8 || (SHIFT == 1 && LAYOUT != kAAOdd) ? 3 : 2;
-    return launch_form<LAYOUT, SHIFT, false, 128, MINB, MINB>(L, a, false);
+    if constexpr (kOneLaunch) {
+      if (a.aux_out) return launch_collide<LAYOUT, SHIFT, false, true, 64, 4>(L, a);
+      if (fused(L, 0)) return launch_step<LAYOUT, SHIFT, 64, 4>(L, a);
+    } else {
+      if (a.aux_out) return launch_collide<LAYOUT, SHIFT, false, true, 128, MINB>(L, a);
+    }
+    return launch_collide<LAYOUT, SHIFT, false, false, 128, MINB>(L, a);
   }
 
   template <int LAYOUT, int VI>
@@ -307,7 +311,7 @@ struct Impl {
     const S* fp = static_cast<const S*>(f);
     C* ap = static_cast<C*>(L.aux);
     C* sp = static_cast<C*>(L.sums);
-    constexpr bool kSums = sizeof(C) == 8;  // as launch_form takes them
+    constexpr bool kSums = sizeof(C) == 8;  // as launch_collide takes them
     if (layout == kPingPong) k_aux<Q, S, C, REP, kPingPong, kSums><<<grid, 256, 0, L.st>>>(fp, ap, sp, G);
     else if (layout == kAAEven) k_aux<Q, S, C, REP, kAAEven, kSums><<<grid, 256, 0, L.st>>>(fp, ap, sp, G);
     else k_aux<Q, S, C, REP, kAAOdd, kSums><<<grid, 256, 0, L.st>>>(fp, ap, sp, G);

@@ -527,7 +527,9 @@ __device__ __forceinline__ typename Codec<S>::W load_word(const S* p) {
 // FP16 collide 3.53 to 3.37 ms). The relaxation uses them with 4-byte storage
 // only (149 x 101 x 67 FP32 deviations in place, a pass of 100 steps: 50.4 ms,
 // 52.7 with scalars); with 16 bits the neighbouring registers they want cost the
-// compiler freedom between pass 2's loads (3.49 ms instead of 3.37).
+// compiler freedom between pass 2's loads (3.49 ms instead of 3.37), as in the
+// in-place LAG form of deviations with a shift field (128^3: 887 us with
+// scalars, 904 with pairs).
 __device__ __forceinline__ float2 pair(float a) { return make_float2(a, a); }
 template <class S>
 __device__ __forceinline__ void unpack_pairs(typename Codec<S>::W w, float2 v[2]) {
@@ -650,11 +652,12 @@ __device__ __forceinline__ bool collide_body(const StepArgs<S, C>& a, const Nbr&
   constexpr int dim = L::kDim;
   // in place (AA) the buffer is written by this kernel: coherent loads
   constexpr bool kCoh = COHF || LAYOUT != kPingPong;
-  constexpr int POL1 = kCoh ? kCoherent : HOLD ? kLast : kKeep;
+  constexpr int POL1 = HOLD ? kLast : kCoh ? kCoherent : kKeep;
   constexpr int POL2 = kCoh ? kCoherent : kLast;
   constexpr bool kLean = lean_coefs<Q, C>;
   constexpr bool kWeighted = sizeof(C) == 8 && REP == kABS;
   constexpr double kWb = L::w(Q - 1);  // the weight that FP64 fluxes carry
+  constexpr bool kLagField = LAGW && SHIFT == 2 && REP == kDEV;
   const int64_t cells = a.G.cells;
 
   W hw[HOLD ? NW : 1][HOLD ? Q : 1];
@@ -662,14 +665,12 @@ __device__ __forceinline__ bool collide_body(const StepArgs<S, C>& a, const Nbr&
   if constexpr (HOLD) {
 #pragma unroll
     for (int m = 0; m < NW; ++m) {
-#pragma unroll
-      for (int l = 0; l < Q; ++l)
-        hw[m][l] = load_word<S, POL1>(a.fin + read_index<Q, LAYOUT, S>(n, V * m, l));
       C sum[V];
 #pragma unroll
       for (int i = 0; i < V; ++i) sum[i] = C(0);
 #pragma unroll
       for (int l = 0; l < Q; ++l) {
+        hw[m][l] = load_word<S, POL1>(a.fin + read_index<Q, LAYOUT, S>(n, V * m, l));
         C v[V];
         unpack_word<S>(hw[m][l], v);
 #pragma unroll
@@ -707,12 +708,11 @@ __device__ __forceinline__ bool collide_body(const StepArgs<S, C>& a, const Nbr&
   cell_terms<Q, S, C, REP, SHIFT>(a, n, rt, A, D,
                                   !kLean ? C(1) : kWeighted ? three_omega * C(kWb) : three_omega,
                                   rho, Sr, Fl, Fv);
-  // cf = omega rho + sigma S = omega rho~ + dt S
-  C cf[kNF];
-#pragma unroll
-  for (int F = 0; F < kNF; ++F)
-    cf[F] = kLean ? a.omega * rt[F] + (a.half_dt + a.half_dt) * Sr[F]
-                  : a.omega * rho[F] + a.sigma * Sr[F];
+  // omega rho + sigma S = omega rho~ + dt S
+  auto coef = [&](int F) -> C {
+    return kLean ? a.omega * rt[F] + (a.half_dt + a.half_dt) * Sr[F]
+                 : a.omega * rho[F] + a.sigma * Sr[F];
+  };
   auto flux = [&](int F, int k) -> C {
     if (has_flux(F)) return kLean ? Fl[F - kK][k] : three_omega * Fl[F - kK][k];
     if (SHIFT && is_v(F)) {
@@ -733,12 +733,13 @@ __device__ __forceinline__ bool collide_body(const StepArgs<S, C>& a, const Nbr&
       vw[l] = HOLD ? hw[HOLD ? m : 0][HOLD ? l : 0]
                    : load_word<S, POL2>(a.fin + read_index<Q, LAYOUT, S>(n, V * m, l));
     if constexpr (V == 1) {
+      const C cf = coef(m);
       C b[3];
 #pragma unroll
       for (int k = 0; k < 3; ++k) b[k] = flux(m, k);
 #pragma unroll
       for (int l = 0; l < Q; ++l) {
-        C t = kWeighted ? C(L::w(l)) * cf[m] : cf[m];
+        C t = kWeighted ? C(L::w(l)) * cf : cf;
         if (fluxed(m)) {
 #pragma unroll
           for (int k = 0; k < dim; ++k) {
@@ -757,12 +758,12 @@ __device__ __forceinline__ bool collide_body(const StepArgs<S, C>& a, const Nbr&
         else
           Codec<S>::store_if(dst, out, valid);
       }
-    } else if constexpr (kLean && sizeof(S) == 4) {
+    } else if constexpr (kLean && sizeof(S) == 4 && !(kLagField && LAYOUT != kPingPong)) {
       float2 c2[2], b[2][3];
 #pragma unroll
       for (int p = 0; p < 2; ++p) {
         const int F = V * m + 2 * p;
-        c2[p] = make_float2(cf[F], cf[F + 1]);
+        c2[p] = make_float2(coef(F), coef(F + 1));
 #pragma unroll
         for (int k = 0; k < 3; ++k) b[p][k] = make_float2(flux(F, k), flux(F + 1, k));
       }
@@ -791,18 +792,20 @@ __device__ __forceinline__ bool collide_body(const StepArgs<S, C>& a, const Nbr&
           WordIO<S>::stw_if(dst, Codec<S>::pack(out), valid);
       }
     } else {
-      C b[V][3];
+      C cf[V], b[V][3];
 #pragma unroll
-      for (int i = 0; i < V; ++i)
+      for (int i = 0; i < V; ++i) {
+        cf[i] = coef(V * m + i);
 #pragma unroll
         for (int k = 0; k < 3; ++k) b[i][k] = flux(V * m + i, k);
+      }
 #pragma unroll
       for (int l = 0; l < Q; ++l) {
         C v[V], out[V];
         Codec<S>::unpack(vw[l], v);
 #pragma unroll
         for (int i = 0; i < V; ++i) {
-          C t = cf[V * m + i];
+          C t = cf[i];
           if (fluxed(V * m + i)) {
 #pragma unroll
             for (int k = 0; k < dim; ++k) {
@@ -827,15 +830,34 @@ __device__ __forceinline__ bool collide_body(const StepArgs<S, C>& a, const Nbr&
 // ---------------------------------------------------------------------------
 // One pass a launch, one thread per cell
 // ---------------------------------------------------------------------------
-// TPB threads a block, registers sized for MINB blocks per SM.
+// The LAG forms of 4-byte storage on D3Q19 take the arguments and the
+// neighbours as copies of their own: the same arithmetic, but the compiler then
+// has pass 2's loads under way earlier (128^3 ping-pong, deviations, us a step:
+// 64 x 4 776 and 759, 128 x 2 823 and 760, shift field 911 and 818). In place
+// only deviations with a shift field gain (937 and 904).
+template <int Q, class S, int LAYOUT, int REP, int SHIFT, bool LAGW>
+constexpr bool kOwnArgs = LAGW && Lattice<Q>::kDim == 3 && sizeof(S) == 4 &&
+                          (LAYOUT == kPingPong || (SHIFT == 2 && REP == kDEV));
+template <int Q, class S, class C, int REP, int LAYOUT, int SHIFT, bool HOLD, bool SUMS, bool LAGW>
+__device__ __forceinline__ bool collide_own(const StepArgs<S, C> a, const Nbr n, bool valid) {
+  return collide_body<Q, S, C, REP, LAYOUT, SHIFT, HOLD, SUMS, LAGW, false, false>(a, n, valid, Plain());
+}
+// TPB threads a block, registers sized for MINB blocks per SM. The 1D and 2D
+// forms ask for the block's size at run time: with the constant the register
+// form under LAG took 1000^2 D2Q9 in 160 us instead of 131 (BF16), 191 instead
+// of 180 (FP32 deviations).
 template <int Q, class S, class C, int REP, int LAYOUT, bool HOLD, int SHIFT, bool LAGW, bool SUMS,
           int TPB, int MINB>
 __global__ void __launch_bounds__(TPB, HOLD ? 1 : MINB) k_collide(const StepArgs<S, C> a) {
-  const int64_t cell = (int64_t)blockIdx.x * TPB + threadIdx.x;
+  const int64_t cell = (int64_t)blockIdx.x * (Lattice<Q>::kDim == 3 ? TPB : blockDim.x) + threadIdx.x;
   const bool valid = cell < a.G.cells;
   const Nbr n = make_nbr(a.G, valid ? cell : a.G.cells - 1);
-  if (collide_body<Q, S, C, REP, LAYOUT, SHIFT, HOLD, SUMS, LAGW, false, false>(a, n, valid, Plain()))
-    atomicOr(a.flag, 1);
+  bool bad;
+  if constexpr (kOwnArgs<Q, S, LAYOUT, REP, SHIFT, LAGW>)
+    bad = collide_own<Q, S, C, REP, LAYOUT, SHIFT, HOLD, SUMS, LAGW>(a, n, valid);
+  else
+    bad = collide_body<Q, S, C, REP, LAYOUT, SHIFT, HOLD, SUMS, LAGW, false, false>(a, n, valid, Plain());
+  if (bad) atomicOr(a.flag, 1);
 }
 
 template <int Q, class S, class C, int REP, int LAYOUT, bool SUMS>
