@@ -173,9 +173,19 @@ int lbnr_set_lagged(lbnr_ctx* ctx, const double* in);
 /* The context's LBNR_DERIV_* mode (-1 for NULL). */
 int lbnr_deriv_mode(const lbnr_ctx* ctx);
 
-/* Synchronises and returns LBNR_ENONFINITE if any step so far produced a
+/* Synchronises and returns LBNR_ETIMEOUT if a device-side wait ran out (the
+ * state is half stepped, steps enqueued after it may have been skipped, and
+ * lbnr_moments, lbnr_constraints, lbnr_get_distributions, lbnr_get_cells and
+ * lbnr_get_lagged return the same code after their copy, until lbnr_init or
+ * lbnr_set_distributions), LBNR_ENONFINITE if any step so far produced a
  * non-finite moment, else LBNR_OK. */
 int lbnr_status(lbnr_ctx* ctx);
+
+/* Bound of the device-side waits of the step that runs both passes in one
+ * launch (default 2 s), in nanoseconds. test_short: test hook, 0 normally; 1
+ * makes its waits expect more work than there is, so that they run out.
+ * Synchronises. Errors: LBNR_EINVAL for a null context or limit_ns <= 0. */
+int lbnr_set_step_wait(lbnr_ctx* ctx, int64_t limit_ns, int32_t test_short);
 
 /* Matter (Sec. "Expansion of flat universe"): a homogeneous perfect fluid at
  * rest in the slice frame, energy density rho(t) = rho0 (t0 / t)^2 (the

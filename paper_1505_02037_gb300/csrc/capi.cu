@@ -367,6 +367,14 @@ int flag_status(lbnr_ctx* c, int flag) {
   return LBNR_OK;
 }
 
+// Ends a read-back of the state: synchronises, and refuses a state that a wait
+// or a consistency check left half stepped. Non-finite values are a state too.
+int finish_readback(lbnr_ctx* c) {
+  int flag = 0;
+  const int rc = read_flag(c, &flag);
+  return rc ? rc : flag_status(c, flag & 6);
+}
+
 }  // namespace
 
 extern "C" {
@@ -657,8 +665,7 @@ int lbnr_get_distributions(lbnr_ctx* c, double* out) {
     CUDA_TRY(c, copy_fields(c, out + (size_t)p * cells, c->L.macro, sizeof(double) * 16 * cells,
                             cudaMemcpyDeviceToHost));
   }
-  CUDA_TRY(c, cudaStreamSynchronize(c->st));
-  return LBNR_OK;
+  return finish_readback(c);
 }
 
 int lbnr_get_cells(lbnr_ctx* c, int64_t n, const int64_t* cells, double* out) {
@@ -679,7 +686,7 @@ int lbnr_get_cells(lbnr_ctx* c, int64_t n, const int64_t* cells, double* out) {
                                 c->st));
     CUDA_TRY(c, cudaStreamSynchronize(c->st));
   }
-  return LBNR_OK;
+  return finish_readback(c);
 }
 
 int lbnr_set_distributions(lbnr_ctx* c, const double* in) {
@@ -708,8 +715,7 @@ int lbnr_get_lagged(lbnr_ctx* c, double* out) {
   CUDA_TRY(c, c->ops->lag_to64(c->L, c->aux[c->steps & 1], d));
   CUDA_TRY(c, cudaMemcpyAsync(out, d, sizeof(double) * 7 * (size_t)c->L.cells,
                               cudaMemcpyDeviceToHost, c->st));
-  CUDA_TRY(c, cudaStreamSynchronize(c->st));
-  return LBNR_OK;
+  return finish_readback(c);
 }
 
 int lbnr_set_lagged(lbnr_ctx* c, const double* in) {
@@ -806,6 +812,15 @@ int lbnr_set_variant(lbnr_ctx* c, int v) {
     CUDA_TRY(c, form_changed(c));
     c->variant = v;
   }
+  return LBNR_OK;
+}
+
+int lbnr_set_step_wait(lbnr_ctx* c, int64_t limit_ns, int32_t test_short) {
+  if (!c || limit_ns <= 0) return fail(c, LBNR_EINVAL, "the wait limit must be positive");
+  CUDA_TRY(c, cudaStreamSynchronize(c->st));
+  c->L.sched.wait_ns = (uint64_t)limit_ns;
+  c->L.sched.quota = c->L.sched.slots + (test_short ? 1u : 0u);
+  CUDA_TRY(c, form_changed(c));
   return LBNR_OK;
 }
 

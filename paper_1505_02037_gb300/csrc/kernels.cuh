@@ -628,18 +628,19 @@ __device__ __forceinline__ void aux_body(const S* __restrict__ f, C* __restrict_
 // the lagged fields of reading R17 are written to a.aux_out. COHF, COHA: the
 // distributions, the planes are written by the same launch, so their loads are
 // coherent (L1 bypassed). valid: the cell is not a clamped one past the end.
-// Hooks: what a caller adds (see Plain).
+// Hooks: what a caller adds (see Plain); a hook that gives up ends the cell before
+// its first store.
 // Returns whether a moment was not finite. The caller reports it after the
 // update pass: a global write between the passes (the flag or aux_out may
 // alias the input as far as the compiler knows) would keep pass 2's loads from
 // being issued ahead of the physics.
 struct Plain {
-  __device__ void before_planes() {}  // runs before the planes are read
+  __device__ bool before_planes() { return true; }  // runs before the planes are read
 };
 template <class Before>
 struct Hooked {
   Before before;
-  __device__ __forceinline__ void before_planes() { before(); }
+  __device__ __forceinline__ bool before_planes() { return before(); }
 };
 template <int Q, class S, class C, int REP, int LAYOUT, int SHIFT, bool HOLD, bool SUMS, bool LAGW,
           bool COHF, bool COHA, class Hooks>
@@ -684,7 +685,7 @@ __device__ __forceinline__ bool collide_body(const StepArgs<S, C>& a, const Nbr&
     for (int m = SUMS ? kAuxWords<S> : 0; m < NW; ++m)
       word_sums<Q, S, C, REP, LAYOUT, POL1>(a.fin, n, m, rt + V * m);
   }
-  hooks.before_planes();
+  if (!hooks.before_planes()) return false;
   if constexpr (SUMS && !HOLD) {
     const C* p = a.aux + n.c;
     const C* q = a.sums + n.c;
@@ -886,8 +887,10 @@ __global__ void __launch_bounds__(256) k_aux(const S* __restrict__ f, C* __restr
 // is complete (one counter a unit). Items are claimed in list order, moment
 // tiles never wait, and a collide tile waits only for moment tiles of items
 // before its own, so the first unfinished item always runs: no wait can outlast
-// the work before it. Every wait is bounded all the same (bit 1 of the flag
-// after ~2 s).
+// the work before it. Every wait is bounded all the same (s.wait_ns, 2 s unless
+// the caller sets another): a warp whose wait runs out stores nothing, sets bit 1
+// of the flag and leaves, and with that bit set the launches behind it leave at
+// once, since this one has not zeroed their counters.
 //
 // A cell's moment tile reads what only the cell's own collide tile writes (in
 // place) or a buffer that the launch does not write (ping-pong).
@@ -919,15 +922,17 @@ __device__ __forceinline__ uint64_t step_clock_ns() {
 template <int Q, class S, class C, int REP, int LAYOUT, int SHIFT, int TPB, int MINB>
 __global__ void __launch_bounds__(TPB, MINB) k_step(const StepArgs<S, C> a, C* aux, C* sums,
                                                      const Schedule s) {
-  constexpr uint64_t kLimitNs = 2000000000ull;
   const uint32_t lane = threadIdx.x & 31u;
   const int64_t cells = a.G.cells;
   unsigned done_to = 0;  // moment units at list positions [0, done_to) are complete
+  // a wait has run out since the state was set; looked at after the first claim,
+  // whose latency covers the load's
+  const int stop = __ldcg(a.flag) & 2;
   for (;;) {
     uint32_t item = 0;
     if (lane == 0) item = atomicAdd(s.cnt, 1u);
     item = __shfl_sync(0xffffffffu, item, 0);
-    if (item >= s.items) break;
+    if (item >= s.items || stop) break;
     const Item t = item_at(s, item);
     uint32_t tile, need;
     if (t.pos < s.units) {
@@ -953,7 +958,7 @@ __global__ void __launch_bounds__(TPB, MINB) k_step(const StepArgs<S, C> a, C* a
       uint64_t t0 = 0;
       while (done_to <= need) {
         const unsigned u = done_to + lane;
-        const bool ok = u > need || ld_acquire(s.cnt + 1 + u) >= s.slots;
+        const bool ok = u > need || ld_acquire(s.cnt + 1 + u) >= s.quota;
         const unsigned open = ~__ballot_sync(0xffffffffu, ok);
         done_to += open ? (unsigned)__ffs((int)open) - 1u : 32u;
         if (done_to > need) {
@@ -963,7 +968,7 @@ __global__ void __launch_bounds__(TPB, MINB) k_step(const StepArgs<S, C> a, C* a
         if (open) {
           const uint64_t now = step_clock_ns();
           if (t0 == 0) t0 = now;
-          if (__shfl_sync(0xffffffffu, (unsigned)(now - t0 > kLimitNs), 0)) {
+          if (__shfl_sync(0xffffffffu, (unsigned)(now - t0 > s.wait_ns), 0)) {
             late = true;
             break;
           }
@@ -971,6 +976,7 @@ __global__ void __launch_bounds__(TPB, MINB) k_step(const StepArgs<S, C> a, C* a
         }
       }
       __syncwarp();
+      return !late;
     };
     const bool bad = collide_body<Q, S, C, REP, LAYOUT, SHIFT, false, true, false, false, true>(
         a, n, valid, Hooked<decltype(before_planes)>{before_planes});

@@ -56,7 +56,10 @@ struct Schedule {
   uint32_t lead;       // list distance between the two passes
   FastDiv fslots, fupu;
   uint32_t items;
+  uint32_t quota;      // finished moment items that complete a unit (slots)
+  uint64_t wait_ns;    // bound of a collide tile's wait
 };
+constexpr uint64_t kWaitNs = 2000000000ull;
 
 // A range of tiles, and a second one.
 struct TileRange {
@@ -177,6 +180,8 @@ inline Schedule make_schedule(uint32_t nx, uint32_t ny, uint32_t nz, int vset,
   s.fslots = make_fastdiv(s.slots);
   s.fupu = make_fastdiv(s.upu);
   s.items = s.slots * (s.units + s.lead);
+  s.quota = s.slots;
+  s.wait_ns = kWaitNs;
   return s;
 }
 

@@ -98,6 +98,7 @@ def library(path: str | None = None):
     L.lbnr_variant_name.restype = ctypes.c_char_p
     L.lbnr_set_variant.argtypes = [vp, ctypes.c_int]
     L.lbnr_variant.argtypes = [vp]
+    L.lbnr_set_step_wait.argtypes = [vp, i64, ctypes.c_int32]
     L.lbnr_set_fluid.argtypes = [vp, ctypes.c_double, ctypes.c_double, ctypes.c_double]
     L.lbnr_set_shift.argtypes = [vp, ctypes.c_double, ctypes.c_double, ctypes.c_double]
     L.lbnr_set_shift_field.argtypes = [vp, vp]
@@ -266,6 +267,10 @@ def lbnr_variant_name(ctx, v: int) -> str:
 
 def lbnr_set_variant(ctx, v: int):
     _check(library().lbnr_set_variant(ctx, v), ctx)
+
+
+def lbnr_set_step_wait(ctx, limit_ns: int, test_short: bool = False):
+    _check(library().lbnr_set_step_wait(ctx, int(limit_ns), int(test_short)), ctx)
 
 
 def lbnr_set_fluid(ctx, rho0: float, w: float, t0: float):
