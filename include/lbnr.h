@@ -109,7 +109,13 @@ int lbnr_create(const lbnr_grid* grid, int vset, double tau, double dx, double d
 
 /* Initial distributions from host fields [16][cells]: the shifted equilibrium
  * f = f_eq(rho0) - (dt/2) w_l S(rho0), with A, D taken from rho0 (the paper
- * does not state its initialisation). Resets the step count to 0. */
+ * does not state its initialisation). Resets the step count to 0.
+ *
+ * Host arrays, here and in lbnr_moments and lbnr_get/set_distributions: one
+ * that lies on 8-byte boundaries in a single page-locked allocation or
+ * registration is read or written by a kernel on the context's stream, which
+ * shares the SMs with whatever other streams run meanwhile (10 to 30 ms for the
+ * 2.1 GB of a 256^3 lattice). Any other array goes through the copy engines. */
 int lbnr_init(lbnr_ctx* ctx, const double* fields);
 
 /* Enqueues n steps on the context's stream (graph-captured two-step cycles).

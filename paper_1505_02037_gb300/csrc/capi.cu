@@ -1,6 +1,7 @@
 // C-ABI of the lbnr library (declared in include/lbnr.h): context set-up,
 // device memory layout, the step loop (CUDA graphs of two-step cycles) and
 // the FP64 monitoring calls.
+#include <cuda.h>
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -13,6 +14,7 @@
 
 #include "../../include/lbnr.h"
 #include "dispatch.h"
+#include "transfer.h"
 
 namespace lbnr {
 
@@ -318,16 +320,37 @@ int build_cycle(lbnr_ctx* c, int parity) {
   return LBNR_OK;
 }
 
-// Device address of `bytes` of page-locked host memory at p, or nullptr.
+// One attribute of a pointer from the driver (the runtime has no call for the
+// extent of an allocation or registration).
+bool pointer_attribute(void* value, CUpointer_attribute what, const void* p) {
+  using Query = CUresult (*)(void*, CUpointer_attribute, CUdeviceptr);
+  static const Query query = [] {
+    void* fn = nullptr;
+    cudaDriverEntryPointQueryResult found;
+    if (cudaGetDriverEntryPointByVersion("cuPointerGetAttribute", &fn, 12000, cudaEnableDefault,
+                                         &found) != cudaSuccess) {
+      (void)cudaGetLastError();
+      return Query(nullptr);
+    }
+    return found == cudaDriverEntryPointSuccess ? reinterpret_cast<Query>(fn) : Query(nullptr);
+  }();
+  return query && query(value, what, (CUdeviceptr)(uintptr_t)p) == CUDA_SUCCESS;
+}
+
+// p, if a kernel may use the `bytes` of page-locked host memory there, or
+// nullptr.
 void* mapped(const void* p, size_t bytes) {
-  cudaPointerAttributes a, b;
-  if (bytes == 0 || cudaPointerGetAttributes(&a, p) != cudaSuccess ||
-      cudaPointerGetAttributes(&b, static_cast<const char*>(p) + bytes - 1) != cudaSuccess) {
+  cudaPointerAttributes a;
+  if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
     (void)cudaGetLastError();
     return nullptr;
   }
-  if (a.type != cudaMemoryTypeHost || b.type != cudaMemoryTypeHost || !a.devicePointer ||
-      static_cast<char*>(b.devicePointer) - static_cast<char*>(a.devicePointer) != (ptrdiff_t)(bytes - 1))
+  CUdeviceptr start = 0;
+  size_t size = 0;
+  if (a.type != cudaMemoryTypeHost || a.devicePointer != p ||
+      !pointer_attribute(&start, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, p) ||
+      !pointer_attribute(&size, CU_POINTER_ATTRIBUTE_RANGE_SIZE, p) ||
+      !kernel_reaches((uintptr_t)p, bytes, (uintptr_t)start, size))
     return nullptr;
   return a.devicePointer;
 }
