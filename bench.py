@@ -711,8 +711,8 @@ def timed_steps(lat, n):
     return e0.elapsed_time(e1)
 
 
-def deriv_mode_records(args, line, fields, sync_ms, sync_col_ms, sync_aux_ms, vset, N, storage,
-                       wave, streaming):
+def deriv_mode_records(args, line, fields, sync_ms, sync_col_ms, sync_aux_ms, sync_launches, vset,
+                       N, storage, wave, streaming):
     """The same workload in the LAG derivative mode (reading R17): the collide
     kernel writes the next step's stencil planes itself, so a step is one
     kernel. Timed like the main run (same steps after the same warm-up)."""
@@ -735,7 +735,8 @@ def deriv_mode_records(args, line, fields, sync_ms, sync_col_ms, sync_aux_ms, vs
         line["roofline"]["hbm"]["peak"]
     out = {
         "sync": {"ms_per_step": sync_ms, "value": cells * 16 / (sync_ms * 1e-3) / 1e6,
-                 "kernels_per_step": 2 if sync_aux_ms else 1, "k_aux_ms": sync_aux_ms, "k_collide_ms": sync_col_ms},
+                 "kernels_per_step": sync_launches, "k_aux_ms": sync_aux_ms,
+                 "k_collide_ms": sync_col_ms},
         "lag": {"ms_per_step": ms, "value": cells * 16 / (ms * 1e-3) / 1e6, "kernels_per_step": 1,
                 "k_collide_ms": col, "launch_form": lat.variants[lat.variant],
                 "collide_hbm_frac": alg / (col * 1e-3) / 1e9 / peak,
@@ -894,19 +895,21 @@ def main():
     cbytes = 8 if storage == "f64" else 4
     alg_collide = cells * (2 * 16 * Q * s + 7 * cbytes)  # f in + f out + stencil planes once
     alg_aux = cells * (7 * Q * s + 7 * cbytes)
-    # a moment pass of its own cannot beat its bytes at twice the copy rate; with
-    # none, the collide launch runs both passes
-    peak_gbs = float(measured_peaks()[0]["hbm_gbs"])
-    one_launch = aux_ms * 1e-3 < alg_aux / (2e9 * peak_gbs)
+    launches = lat.launches_per_step
+    one_launch = launches == 1  # both passes in it: the first interval holds no kernel
     if one_launch:
         col_ms, aux_ms = col_ms + aux_ms, 0.0
+    kernel = ("k_collide" if not one_launch else
+              "k_lanes" if form.startswith("lanes") else "k_step")
     peaks, peak_kind = measured_peaks()
     # burst figure: the kernel is timed as one launch of a few milliseconds
     peak = float(peaks["hbm_gbs"])
     achieved = alg_collide / (col_ms * 1e-3) / 1e9
-    tkey = f"k_collide:{args.workload}:{form}"
+    tkey = f"{kernel}:{args.workload}:{form}"
     traffic = traffic_for(tkey, cells)
-    hbm_roofline = {"bound": "hbm", "kernel": "k_collide (fused collide-and-stream)",
+    hbm_roofline = {"bound": "hbm",
+                    "kernel": kernel + (" (both passes of the step)" if one_launch
+                                        else " (fused collide-and-stream)"),
                     "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                     "peak_source": f"hbm_gbs of {peak_kind}",
                     "algorithmic_bytes_per_cell": alg_collide / cells,
@@ -946,7 +949,7 @@ def main():
         "step_algorithmic_hbm_frac": (alg_collide + (0 if one_launch else alg_aux)) / (ms_max / args.steps * 1e-3)
                                      / 1e9 / peak,
         "constraint_monitor_ms_per_call": monitor_ms,
-        "gpu_launches": (1 if one_launch else 2) * args.steps,
+        "gpu_launches": launches * args.steps,
         "launch_form": form,
         "autotune_ms_per_collide": tuning,
         "clocks": clk.summary(),
@@ -982,7 +985,8 @@ def main():
         lat.close()
         del lat
         line["deriv_modes"] = deriv_mode_records(args, line, fields, ms_max / args.steps, col_ms,
-                                                 aux_ms, vset, N, storage, wave, streaming)
+                                                 aux_ms, launches, vset, N, storage, wave,
+                                                 streaming)
         if storage in ("f32", "dev_f32") and wave == "gauge" and direction == "x":
             line["precision_one_crossing"] = precision_records(args, N, local)
 

@@ -250,6 +250,11 @@ const char* lbnr_variant_name(const lbnr_ctx* ctx, int variant);
 int lbnr_set_variant(lbnr_ctx* ctx, int variant);
 int lbnr_variant(const lbnr_ctx* ctx);
 
+/* Kernel launches of one step as the context stands: 1 where both passes share
+ * a launch and under LAG, 2 where the moment pass is a launch of its own, and
+ * one more with a fluid, whose clock is advanced by a launch. -1 for NULL. */
+int lbnr_launches_per_step(const lbnr_ctx* ctx);
+
 /* Steps taken since lbnr_init; Q of the velocity set; the streaming pattern
  * chosen (LBNR_STREAM_PINGPONG or LBNR_STREAM_AA). */
 int64_t lbnr_steps_done(const lbnr_ctx* ctx);

@@ -847,6 +847,12 @@ int lbnr_set_step_wait(lbnr_ctx* c, int64_t limit_ns, int32_t test_short) {
   return LBNR_OK;
 }
 
+int lbnr_launches_per_step(const lbnr_ctx* c) {
+  if (!c) return -1;
+  const LaunchCtx L = step_ctx(c, c->steps);
+  return (lagged(c) || c->ops->fused(L, c->variant) ? 1 : 2) + (c->L.clock ? 1 : 0);
+}
+
 int lbnr_variant(const lbnr_ctx* c) { return c ? c->variant : -1; }
 
 int64_t lbnr_steps_done(const lbnr_ctx* c) { return c ? c->steps : -1; }
