@@ -1,13 +1,13 @@
-"""Per-cell DRAM traffic of a collide kernel, from an ncu capture, as an
+"""Per-cell DRAM traffic of a step's kernel, from an ncu capture, as an
 entry of the traffic table the benchmark reads (profiles/traffic.json).
 
 Run right after the capture, on the machine that made it:
 
   ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum,gpu__time_duration.sum \\
-      --clock-control none -k regex:k_collide -s 2 -c 1 --csv --log-file cap.csv \\
-      python -m paper_1505_02037_gb300.profile_step --storage f32 --n 128 --variant P1-reread
+      --clock-control none -k "regex:k_collide|k_step" -s 2 -c 1 --csv --log-file cap.csv \\
+      python -m paper_1505_02037_gb300.profile_step --storage f32 --n 128 --variant P1-reread-64x4
   python -m paper_1505_02037_gb300.traffic_table cap.csv \\
-      --key k_collide:gauge3d-256-f32:P1-reread --cells 2097152 --out traffic_new.json \\
+      --key k_step:gauge3d-256-f32:P1-reread-64x4 --cells 2097152 --out traffic_new.json \\
       --captured-on "D3Q19 FP32 128^3 gauge wave, one launch" --command "<the ncu line>"
 
 The entry records the hash of the kernel sources as they are when this
@@ -27,14 +27,17 @@ import sys
 HERE = os.path.dirname(os.path.abspath(__file__))
 
 # Sources the collide-and-stream kernels of the 3D lattice are built from.
-COLLIDE_SOURCES = ("collide_tma.cuh", "dispatch.h", "instantiate.cuh",
-                   "kernels.cuh", "lattice.cuh", "physics.cuh", "inst_q19_s0.cu",
+COLLIDE_SOURCES = ("collide_tma.cuh", "dispatch.h", "instantiate.cuh", "kernels.cuh",
+                   "lanes.cuh", "lattice.cuh", "physics.cuh", "schedule.h", "inst_q19_s0.cu",
                    "inst_q19_s1.cu", "inst_q19_s2.cu", "inst_q19_s3.cu", "inst_q19_s4.cu")
 # Sources the 37-field collide kernel is built from.
 AD_SOURCES = ("ad.cuh", "ad_q19_f32.cu", "dispatch.h", "kernels.cuh", "lattice.cuh",
-              "physics.cuh")
+              "physics.cuh", "schedule.h")
 # Sources of the batched ensemble kernel.
-BATCH_SOURCES = ("batch.cu", "dispatch.h", "kernels.cuh", "lattice.cuh", "physics.cuh")
+BATCH_SOURCES = ("batch.cu", "dispatch.h", "kernels.cuh", "lattice.cuh", "physics.cuh",
+                 "schedule.h")
+# Kernels that take a step, the first one found in a capture.
+STEP_KERNELS = ("k_step", "k_lanes", "k_collide")
 
 
 def source_hash(files=COLLIDE_SOURCES) -> str:
@@ -69,7 +72,7 @@ def main(argv=None):
     p = argparse.ArgumentParser()
     p.add_argument("csv")
     p.add_argument("--key", required=True)
-    p.add_argument("--kernel", default="k_collide")
+    p.add_argument("--kernel", default=None, help="part of its name (default: the step's kernel)")
     p.add_argument("--cells", type=int, required=True)
     p.add_argument("--sources", default="collide", choices=["collide", "ad", "batch"])
     p.add_argument("--captured-on", required=True)
@@ -78,9 +81,10 @@ def main(argv=None):
     p.add_argument("--flops-per-cell", type=float, default=None)
     a = p.parse_args(argv)
     files = {"collide": COLLIDE_SOURCES, "ad": AD_SOURCES, "batch": BATCH_SOURCES}[a.sources]
-    rows = read_ncu_csv(a.csv, a.kernel)
+    names = (a.kernel,) if a.kernel else STEP_KERNELS
+    rows = next((r for r in (read_ncu_csv(a.csv, n) for n in names) if r), None)
     if not rows:
-        print(f"no launch of {a.kernel} in {a.csv}")
+        print(f"no launch of {' or '.join(names)} in {a.csv}")
         return 2
     m = rows[-1]
     rd = m["dram__bytes_read.sum"] / a.cells
