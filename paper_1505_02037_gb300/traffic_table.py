@@ -31,8 +31,8 @@ COLLIDE_SOURCES = ("collide_tma.cuh", "dispatch.h", "instantiate.cuh", "kernels.
                    "lanes.cuh", "lattice.cuh", "physics.cuh", "schedule.h", "inst_q19_s0.cu",
                    "inst_q19_s1.cu", "inst_q19_s2.cu", "inst_q19_s3.cu", "inst_q19_s4.cu")
 # Sources the 37-field collide kernel is built from.
-AD_SOURCES = ("ad.cuh", "ad_q19_f32.cu", "dispatch.h", "kernels.cuh", "lattice.cuh",
-              "physics.cuh", "schedule.h")
+AD_SOURCES = ("ad.cuh", "ad_q19_f32.cu", "collide_tma.cuh", "dispatch.h", "kernels.cuh",
+              "lattice.cuh", "physics.cuh", "schedule.h")
 # Sources of the batched ensemble kernel.
 BATCH_SOURCES = ("batch.cu", "dispatch.h", "kernels.cuh", "lattice.cuh", "physics.cuh",
                  "schedule.h")
