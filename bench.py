@@ -316,11 +316,22 @@ ENSEMBLE_SEED = 150502037
 
 
 # FP64 flops per cell of the D3Q19 FP64 collide (dadd + dmul + 2 dfma thread
-# instructions per cell, counted by ncu on the 64^3 gauge wave); used when
-# the traffic table holds no count taken on the current sources
+# instructions per cell, counted by ncu on the 64^3 gauge wave) before its
+# sources were shortened. A record only: a rate made from it and today's time is
+# a speed-up, not the share of the FP64 pipe that is in use.
 FP64_FLOPS_PER_CELL = 2948.0
-FP64_FLOPS_SOURCE = ("ncu counts of the FP64 collide (64^3 gauge wave), last taken on the "
-                     "tile-blocked layout; the traffic table holds none for these sources")
+
+
+def fp64_alu(key, cells, ms, peak_tflops):
+    """The FP64 operations' rate of a kernel launch of `ms` milliseconds and its
+    fraction of the measured FMA rate, from the counts that the traffic table
+    holds for these sources; None without such a count."""
+    flops = profile_entry(key, "fp64_flops_per_cell")
+    if flops is None:
+        return None
+    achieved = flops * cells / (ms * 1e-3) / 1e12
+    return {"flops_per_cell": flops, "achieved_tflops": achieved, "frac": achieved / peak_tflops,
+            "flops_source": "ncu counts on the current sources (profiles/traffic.json)"}
 
 E2E_REPEATS = 3
 
@@ -778,18 +789,12 @@ def precision_records(args, N, device_index):
         if storage == "f64":
             # the FP64 step is bound by the FP64 pipe: its collide kernel's
             # flops (ncu count per cell) against the rate measured here
-            flops = profile_entry(f"k_collide:gauge3d-{N}-f64:{rec['launch_form']}",
-                                  "fp64_flops_per_cell")
-            source = "ncu counts on the current sources (profiles/traffic.json)"
-            if flops is None:
-                flops, source = FP64_FLOPS_PER_CELL, FP64_FLOPS_SOURCE
             _, col = lat.step_timed(4)
             peak = lbnr.lbnr_fp64_fma_rate(lat.stream)
             rec["collide_ms"] = col / 4
             rec["fp64_peak_tflops_measured"] = peak
-            ach = flops * cells / (col / 4 * 1e-3) / 1e12
-            rec["alu"] = {"flops_per_cell": flops, "flops_source": source, "achieved_tflops": ach,
-                          "frac": ach / peak}
+            rec["alu"] = fp64_alu(f"k_collide:gauge3d-{N}-f64:{rec['launch_form']}", cells, col / 4,
+                                  peak)
         if finite:
             rec["err_vs_analytic"] = float(np.abs(m - exact).max() / A)
             if ref is None:
@@ -915,20 +920,18 @@ def main():
                     "algorithmic_bytes_per_cell": alg_collide / cells,
                     "avg_launch_ms": col_ms, "traffic": traffic}
     roofline = hbm_roofline
-    flops = profile_entry(tkey, "fp64_flops_per_cell") if storage == "f64" else None
-    flops_source = "ncu counts on the current sources (profiles/traffic.json)"
-    if storage == "f64" and flops is None:
-        flops, flops_source = FP64_FLOPS_PER_CELL, FP64_FLOPS_SOURCE
-    if flops is not None:
+    if storage == "f64":
         # FP64 is bound by the FP64 pipe: its peak is the rate a register
         # FMA-chain kernel sustains on this GPU, measured here
         fp64_peak = lbnr.lbnr_fp64_fma_rate(lat.stream)
-        ach = flops * cells / (col_ms * 1e-3) / 1e12
+        alu = fp64_alu(tkey, cells, col_ms, fp64_peak) or {}
         roofline = {"bound": "alu", "kernel": "k_collide (fused collide-and-stream, FP64)",
-                    "achieved": ach, "peak": fp64_peak, "unit": "TFLOP/s", "frac": ach / fp64_peak,
+                    "achieved": alu.get("achieved_tflops"), "peak": fp64_peak, "unit": "TFLOP/s",
+                    "frac": alu.get("frac"),
                     "peak_source": "measured in this run: FP64 FMA chains at full occupancy "
                                    "(lbnr_fp64_fma_rate)",
-                    "flops_per_cell": flops, "flops_source": flops_source,
+                    "flops_per_cell": alu.get("flops_per_cell"),
+                    "flops_source": alu.get("flops_source", "no count on the current sources"),
                     "avg_launch_ms": col_ms, "traffic": traffic, "hbm": hbm_roofline}
 
     value = units_all / (ms_max * 1e-3) / 1e6
