@@ -233,6 +233,10 @@ int lbnr_set_shift(lbnr_ctx* ctx, double bx, double by, double bz);
  * allocated. */
 int lbnr_set_shift_field(lbnr_ctx* ctx, const double* beta);
 
+/* 1 if the context carries a constant shift or a shift field (its steps then
+ * run the shift's one launch form), 0 if not, -1 for NULL. */
+int lbnr_has_shift(const lbnr_ctx* ctx);
+
 /* Launch forms of the collide kernel available for this context's set and
  * storage (all give the same results within rounding): their number, a short
  * name, and the selection (default: form 0, for small FP64 ping-pong lattices

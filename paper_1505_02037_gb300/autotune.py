@@ -15,7 +15,13 @@ _cache: dict = {}
 def tune(lat, steps_per_trial: int = 4, trials: int = 2, verbose: bool = False) -> dict:
     """Chooses the fastest launch form for `lat` (a lbnr.Lattice that has
     been initialised). The trial steps advance the simulation like any other
-    steps. Returns {name: ms per step}."""
+    steps. Returns {name: ms per step}.
+
+    A lattice with a shift runs the one form that carries the shift terms,
+    whichever is selected: it is left as it is, and nothing is kept for its
+    key, which unshifted lattices share."""
+    if lat.has_shift:
+        return {}
     key = (lat.vset, lat.storage, lat.streaming, lat.shape, lat.deriv_mode)
     names = lat.variants
     if key in _cache:

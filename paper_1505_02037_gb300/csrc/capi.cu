@@ -847,6 +847,8 @@ int lbnr_set_step_wait(lbnr_ctx* c, int64_t limit_ns, int32_t test_short) {
   return LBNR_OK;
 }
 
+int lbnr_has_shift(const lbnr_ctx* c) { return c ? c->L.shift_on : -1; }
+
 int lbnr_launches_per_step(const lbnr_ctx* c) {
   if (!c) return -1;
   const LaunchCtx L = step_ctx(c, c->steps);

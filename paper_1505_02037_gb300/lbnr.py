@@ -99,6 +99,7 @@ def library(path: str | None = None):
     L.lbnr_set_variant.argtypes = [vp, ctypes.c_int]
     L.lbnr_variant.argtypes = [vp]
     L.lbnr_launches_per_step.argtypes = [vp]
+    L.lbnr_has_shift.argtypes = [vp]
     L.lbnr_set_step_wait.argtypes = [vp, i64, ctypes.c_int32]
     L.lbnr_set_fluid.argtypes = [vp, ctypes.c_double, ctypes.c_double, ctypes.c_double]
     L.lbnr_set_shift.argtypes = [vp, ctypes.c_double, ctypes.c_double, ctypes.c_double]
@@ -503,6 +504,10 @@ class Lattice:
     def set_lagged(self, prev):
         lbnr_set_lagged(self.ctx, np.ascontiguousarray(np.asarray(prev, dtype=np.float64)
                                                        .reshape(7, self.cells)))
+
+    @property
+    def has_shift(self):
+        return library().lbnr_has_shift(self.ctx) == 1
 
     @property
     def launches_per_step(self):
