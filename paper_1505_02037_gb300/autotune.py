@@ -9,13 +9,21 @@ runs, CUDA events per kernel) and keeps the fastest. Results are cached per
 """
 from __future__ import annotations
 
+from .lbnr import LBNR_STREAM_PINGPONG
+
+# Above this many cells the forms with several lanes per cell are not tried: they
+# fill the schedulers at 1500 to 8000 cells and fall behind for good (20^3 D3Q19
+# 77 against 72 us a step, 64^3 2.4 and 3.2 times the time). In place they are
+# form 0 under another name.
+LANES_MAX_CELLS = 16384
+
 _cache: dict = {}
 
 
 def tune(lat, steps_per_trial: int = 4, trials: int = 2, verbose: bool = False) -> dict:
     """Chooses the fastest launch form for `lat` (a lbnr.Lattice that has
     been initialised). The trial steps advance the simulation like any other
-    steps. Returns {name: ms per step}.
+    steps. Returns {name: ms per step} of the forms tried.
 
     A lattice with a shift runs the one form that carries the shift terms,
     whichever is selected: it is left as it is, and nothing is kept for its
@@ -29,6 +37,9 @@ def tune(lat, steps_per_trial: int = 4, trials: int = 2, verbose: bool = False) 
         return {}
     times = {}
     for v, name in enumerate(names):
+        if name.startswith("lanes") and (lat.streaming != LBNR_STREAM_PINGPONG
+                                         or lat.cells > LANES_MAX_CELLS):
+            continue
         lat.set_variant(v)
         lat.step_timed(2)  # first launch pays for set-up
         best = float("inf")
@@ -38,7 +49,7 @@ def tune(lat, steps_per_trial: int = 4, trials: int = 2, verbose: bool = False) 
         times[name] = best
         if verbose:
             print(f"  {name}: {times[name]:.3f} ms per step")
-    best = min(range(len(names)), key=lambda v: times[names[v]])
+    best = names.index(min(times, key=times.get))
     lat.set_variant(best)
     _cache[key] = best
     return times

@@ -43,3 +43,13 @@ def test_shifted_lattice_is_left_alone():
     assert autotune.tune(a) == {} and a.variant == 0 and a.steps == 0
     b = Stand({"x": 1.0, "y": 2.0})
     assert autotune.tune(b) and b.variant == 0
+
+
+@pytest.mark.parametrize("shape,streaming,tried", [
+    ((20, 20, 20), 1, True), ((16384, 1, 1), 1, True), ((16385, 1, 1), 1, False),
+    ((64, 64, 64), 1, False), ((20, 20, 20), 2, False)])
+def test_lane_forms_are_tried_where_they_can_win(shape, streaming, tried):
+    a = Stand({"P1-reread": 2.0, "lanes16": 3.0, "lanes8": 1.0}, streaming=streaming, shape=shape)
+    times = autotune.tune(a)
+    assert ("lanes16" in times) == tried and ("lanes8" in times) == tried
+    assert a.variant == (2 if tried else 0)
