@@ -328,7 +328,9 @@ typedef struct {
 typedef struct {
   int32_t storage;      /* LBNR_F64 ... LBNR_DEV_F16, for every run */
   int32_t block;        /* threads per block: 128 or 256 (default 256) */
-  int32_t ctas_per_sm;  /* resident blocks per SM; 0 = as many as fit */
+  int32_t ctas_per_sm;  /* resident blocks per SM; 0 = as many as fit; of blocks
+                           of 256, one or two by storage, cells and how evenly
+                           the runs divide */
   int32_t sources_on;   /* 1 normally; 0 drops every source */
   void* cuda_stream;    /* cudaStream_t; NULL = a stream of the batch's own */
   int64_t wait_limit_ns; /* bound of every device-side barrier wait (2 s) */

@@ -57,9 +57,9 @@ def tune(lat, steps_per_trial: int = 4, trials: int = 2, verbose: bool = False) 
 
 def batch_shapes(sm_resident_max: int = 4):
     """(threads per block, blocks per SM) pairs the batched kernel accepts:
-    blocks of 256 threads at up to 255 registers (one per SM), blocks of 128
-    at up to 168 registers (one to three per SM) or at up to 128 (four)."""
-    shapes = [(256, 1), (128, 1), (128, 2), (128, 3), (128, 4)]
+    blocks of 256 threads at up to 255 registers (one per SM) or 128 (two),
+    blocks of 128 at up to 168 registers (one to three per SM) or 128 (four)."""
+    shapes = [(256, 1), (256, 2), (128, 1), (128, 2), (128, 3), (128, 4)]
     return [s for s in shapes if s[1] <= sm_resident_max]
 
 

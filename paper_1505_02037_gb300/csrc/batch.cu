@@ -5,7 +5,7 @@
 // with the equilibria and sources of Eqs. alfa-ekstsor): a moment pass for
 // the derivative stencil, then the fused collide-and-stream pass.
 //
-// Plan (host): a run's cost is cells x steps x Q. With W resident CTAs and
+// Plan (host): a run's cost is cells x steps x (Q + 8). With W resident CTAs and
 // an even share L = total / W, a run costing more than L gets a team of
 // ceil(cost / L) CTAs of its own. The work list holds one entry per team
 // member first, then every other run, longest first; each CTA claims the
@@ -40,6 +40,7 @@
 #include <vector>
 
 #include "../../include/lbnr.h"
+#include "batch_plan.h"
 #include "dispatch.h"
 #include "kernels.cuh"
 
@@ -50,12 +51,6 @@ namespace {
 // run costs: the sources and fluxes. Without it 1D runs got too few blocks and
 // finished last (32 uneven runs, 256 x 1: 68.6 ms at 0, 67.9 at 4, 58.9 at 8, 58.6 at 20).
 constexpr double kCellCost = 8;
-// Between these many cells in all runs, blocks of 256 are sized for two per SM
-// where the caller leaves the number open: fewer, and a step waits for one
-// block's chain of passes, which more registers shorten; more, and the runs
-// miss the L2. ms, one against two per SM (SYNC): 31e3 cells 4.20 / 5.50, 230e3
-// 33.4 / 30.1, 1.7e6 125.5 / 113.0, 6.7e6 844 / 774, 18e6 2029 / 2396.
-constexpr int64_t kFewCells = 120000, kManyCells = 10000000;
 
 struct BatchRun {
   void* f[2];
@@ -260,10 +255,10 @@ void* batch_kernel_form(int storage) {
   }
 }
 
-// Form for a block size and a requested number of blocks per SM (0: the
-// form's own maximum, chosen by the cells of all runs).
-int form_for(int block, int per_sm, int64_t cells) {
-  if (block == 256) return per_sm == 1 || (per_sm == 0 && (cells < kFewCells || cells > kManyCells)) ? 0 : 3;
+// Form for a block size and a number of blocks per SM (0: as many as fit;
+// blocks of 256 take one form for one and another for two).
+int form_for(int block, int per_sm) {
+  if (block == 256) return per_sm == 1 ? 0 : 3;
   return per_sm == 4 ? 2 : 1;
 }
 
@@ -313,6 +308,7 @@ struct lbnr_batch {
   int grid = 0, block = 256, form = 0;
   std::vector<Assign> work;
   std::vector<int> team;   // blocks per run in the current plan (0: not stepped)
+  std::vector<double> cost;  // and what each run costs there
   size_t work_cap = 0;
   Assign* h_work = nullptr;  // pinned staging of the work list
   int* h_nwork = nullptr;
@@ -351,6 +347,7 @@ void make_plan(lbnr_batch* b, int workers, const std::vector<char>& live) {
                  : 0.0;
     total += cost[r];
   }
+  b->cost = cost;
   const double share = total / std::max(workers, 1);
   std::vector<int> team(R, 1);
   int big = 0;
@@ -415,12 +412,51 @@ int live_runs(lbnr_batch* b, std::vector<char>& live) {
   return LBNR_OK;
 }
 
+// Blocks of 256 per SM where the caller leaves the number open. Leaves the plan
+// as it was.
+int choose_per_sm(lbnr_batch* b, int sms, const std::vector<char>& live) {
+  const int R = (int)b->runs.size();
+  const std::vector<Assign> work = b->work;
+  const std::vector<int> team = b->team;
+  const std::vector<double> cost = b->cost;
+  const int grid = b->grid, block = b->block;
+  b->block = 256;
+  std::vector<int64_t> cells(R);
+  double even[2], total = 0, single = 0;
+  int64_t all = 0, all_2d = 0;
+  for (int r = 0; r < R; ++r) cells[r] = b->runs[r].grid.nx * b->runs[r].grid.ny;
+  for (int per_sm = 2; per_sm >= 1; --per_sm) {  // the plan of one last: it is looked at below
+    make_plan(b, sms * per_sm, live);
+    even[per_sm - 1] = imbalance(b->cost, cells, b->team, sms * per_sm, b->block);
+  }
+  for (int r = 0; r < R; ++r) {
+    if (b->team[r] == 0) continue;
+    all += cells[r];
+    if (b->runs[r].vset == LBNR_D2Q9) all_2d += cells[r];
+    total += b->cost[r];
+    if (b->team[r] == 1) single += b->cost[r];
+  }
+  const size_t bytes = b->opts.storage == LBNR_F64 ? 8
+                       : b->opts.storage == LBNR_F32 || b->opts.storage == LBNR_DEV_F32 ? 4 : 2;
+  b->work = work;
+  b->team = team;
+  b->cost = cost;
+  b->grid = grid;
+  b->block = block;
+  return two_per_sm(bytes, all, all_2d, total > 0 ? single / total : 0.0, even[0], even[1]) ? 2 : 1;
+}
+
 int configure(lbnr_batch* b, int block, int ctas_per_sm) {
   if (block != 128 && block != 256) return bfail(b, LBNR_EINVAL, "block must be 128 or 256");
   if (ctas_per_sm < 0 || ctas_per_sm > 4) return bfail(b, LBNR_EINVAL, "ctas_per_sm must be 0..4");
-  int64_t cells = 0;
-  for (const lbnr_run_desc& d : b->runs) cells += d.grid.nx * d.grid.ny;
-  const int form = form_for(block, ctas_per_sm, cells);
+  int dev = 0, sms = 0;
+  BTRY(b, cudaGetDevice(&dev));
+  BTRY(b, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  std::vector<char> live;
+  int rc = live_runs(b, live);
+  if (rc) return rc;
+  if (block == 256 && ctas_per_sm == 0) ctas_per_sm = choose_per_sm(b, sms, live);
+  const int form = form_for(block, ctas_per_sm);
   void* kern = batch_kernel(b->opts.storage, form, b->opts.deriv_mode);
   // the kernel uses no shared memory to speak of: give the SM's unified
   // cache to L1
@@ -428,9 +464,6 @@ int configure(lbnr_batch* b, int block, int ctas_per_sm) {
   int occ = 0;
   BTRY(b, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, block, 0));
   if (occ < 1) return bfail(b, LBNR_ECUDA, "batched kernel cannot be resident");
-  int dev = 0, sms = 0;
-  BTRY(b, cudaGetDevice(&dev));
-  BTRY(b, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   const int per_sm = ctas_per_sm > 0 ? std::min(ctas_per_sm, occ) : occ;
   const int workers = sms * per_sm;
   // work list buffers: at most one entry per CTA for team members plus one
@@ -452,9 +485,6 @@ int configure(lbnr_batch* b, int block, int ctas_per_sm) {
   }
   b->block = block;
   b->form = form;
-  std::vector<char> live;
-  int rc = live_runs(b, live);
-  if (rc) return rc;
   make_plan(b, workers, live);
   return upload_plan(b);
 }

@@ -34,8 +34,8 @@ COLLIDE_SOURCES = ("collide_tma.cuh", "dispatch.h", "instantiate.cuh", "kernels.
 AD_SOURCES = ("ad.cuh", "ad_q19_f32.cu", "collide_tma.cuh", "dispatch.h", "kernels.cuh",
               "lattice.cuh", "physics.cuh", "schedule.h")
 # Sources of the batched ensemble kernel.
-BATCH_SOURCES = ("batch.cu", "dispatch.h", "kernels.cuh", "lattice.cuh", "physics.cuh",
-                 "schedule.h")
+BATCH_SOURCES = ("batch.cu", "batch_plan.h", "dispatch.h", "kernels.cuh", "lattice.cuh",
+                 "physics.cuh", "schedule.h")
 # Kernels that take a step, the first one found in a capture.
 STEP_KERNELS = ("k_step", "k_lanes", "k_collide")
 
