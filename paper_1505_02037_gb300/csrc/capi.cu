@@ -198,11 +198,15 @@ int validate(const lbnr_grid* g, int vset, const lbnr_opts* o) {
   return LBNR_OK;
 }
 
-// The work list of the lattice's SYNC step. Its counters, of the even and the
-// odd step, take the front of the staging area; a lattice whose counters would
-// fill more than half of that (2.6e8 cells) runs one pass a launch.
-Schedule schedule_for(const lbnr_grid* g, int vset) {
-  Schedule s = make_schedule((uint32_t)g->nx, (uint32_t)g->ny, (uint32_t)g->nz, vset);
+// The work list of the lattice's SYNC step, empty where both passes do not share
+// a launch. Its counters, of the even and the odd step, take the front of the
+// staging area; a lattice whose counters would fill more than half of that
+// (2.6e8 cells) runs one pass a launch.
+Schedule schedule_for(const lbnr_grid* g, int vset, const lbnr_opts* o) {
+  Schedule s = {};
+  if (!one_launch_step(q_of(vset), storage_bytes(o->storage)) || o->deriv_mode == LBNR_DERIV_LAG)
+    return s;
+  s = make_schedule((uint32_t)g->nx, (uint32_t)g->ny, (uint32_t)g->nz, vset);
   if (2 * align256(4ull * (1 + s.units)) > kStageBytes / 2) s.units = 0;
   return s;
 }
@@ -521,14 +525,13 @@ int lbnr_create(const lbnr_grid* grid, int vset, double tau, double dx, double d
   // the moment pass's other two planes share the FP64 field planes, which no
   // step keeps anything in
   L.sums = L.macro;
-  L.sched = schedule_for(grid, vset);
+  L.sched = schedule_for(grid, vset, opts);
   const uint64_t counters = L.sched.units ? align256(4ull * (1 + L.sched.units)) : 0;
   c->counters_bytes = 2 * counters;
   c->counters[0] = reinterpret_cast<uint32_t*>(b + Ly.stage);
   c->counters[1] = reinterpret_cast<uint32_t*>(b + Ly.stage + counters);
   L.stage = b + Ly.stage + c->counters_bytes;
   L.st = c->st;
-  L.block = 128;
   L.clock = nullptr;
   L.fluid_P0 = L.fluid_t0 = L.fluid_P_now = 0;
   L.beta[0] = L.beta[1] = L.beta[2] = 0;

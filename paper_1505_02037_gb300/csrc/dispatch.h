@@ -10,6 +10,9 @@
 namespace lbnr {
 
 constexpr uint64_t kStageBytes = 1ull << 20;
+// Sets and storage whose SYNC step runs both passes in one launch (k_step says
+// why the others do not).
+constexpr bool one_launch_step(int Q, size_t storage_bytes) { return Q == 19 && storage_bytes == 4; }
 constexpr int64_t kTile = 32;  // cells per tile of the tile-blocked distribution layout
 
 struct LaunchCtx {
@@ -29,7 +32,6 @@ struct LaunchCtx {
   void* stage;      // staging area for sampled transfers (kStageBytes)
   int* flag;        // non-finite flag
   cudaStream_t st;
-  int block;        // threads per block of the collide kernel
   // Matter (perfect fluid at rest): pressure P0 (t0/t)^2 at t = t0 + n dt;
   // clock points at the device step counter n (nullptr: vacuum), P_now is
   // the pressure at the state the FP64 moment calls read.

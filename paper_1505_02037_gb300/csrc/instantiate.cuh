@@ -112,7 +112,7 @@ struct Impl {
   }
 
   // Storage whose SYNC step can run both passes in one launch (k_step).
-  static constexpr bool kOneLaunch = Q == 19 && sizeof(S) == 4;
+  static constexpr bool kOneLaunch = one_launch_step(Q, sizeof(S));
   // Whether the step of this variant runs the moment pass itself.
   static bool fused(const LaunchCtx& L, int variant) {
     const VariantSpec& x = VT::v[variant >= 0 && variant < VT::n ? variant : 0];

@@ -443,8 +443,8 @@ __device__ __forceinline__ void bm_flux(const T al, const T g[6], const T V[3], 
     bm_flux_plain<T, dim>(al, g, V, A, D, F);
     return;
   }
-  T gi[6], idet;
-  invert_sym3(g, gi, idet);
+  T gi[6];
+  invert_sym3(g, gi);
   const T ah = T(0.5) * al;
   T e[3], ga[6];
 #pragma unroll
