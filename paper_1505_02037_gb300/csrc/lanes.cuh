@@ -33,6 +33,9 @@ namespace lbnr {
 // cells 11.3, 12.3, 25.6; 2500 19.4, 14.4, 25.6; 6000 36.9, 24.6, 25.6. D2Q9 32^2
 // 14.3, 17.4, 45.1; 70^2 41.0, 31.8, 46.1; 90^2 61.4, 45.2, 46.1. D3Q19 8^3 17.4,
 // 22.6, 69.7; 12^3 22.6, 24.6, 71.7; 16^3 47.1, 34.8, 71.7; 20^3 87.1, 77.3, 71.7.
+// LAG crosses at much the same sizes: D1Q3 1500 12.3, 12.3, 21.5; 5500 34.8, 23.6,
+// 22.5; D2Q9 41^2 15.4, 15.4, 40.0; 89^2 56.4, 40.0, 40.0; D3Q19 2000 cells 21.5,
+// 19.5, 62.5; 19^3 65.3, 44.5, 62.5.
 template <int Q>
 constexpr int lanes_for(int64_t cells) {
   return cells <= (Q == 3 ? 1500 : Q == 9 ? 1700 : 2000) ? 16
