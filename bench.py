@@ -330,7 +330,12 @@ def fp64_alu(key, cells, ms, peak_tflops):
     if flops is None:
         return None
     achieved = flops * cells / (ms * 1e-3) / 1e12
-    return {"flops_per_cell": flops, "achieved_tflops": achieved, "frac": achieved / peak_tflops,
+    # the pipe takes an addition or a product as long as a fused multiply-add,
+    # which counts as two flops: its use goes by instructions
+    n = profile_entry(key, "fp64_instructions_per_cell")
+    return {"pipe_frac": None if n is None else
+            n * cells / (ms * 1e-3) / (peak_tflops * 1e12 / 2),
+            "flops_per_cell": flops, "achieved_tflops": achieved, "frac": achieved / peak_tflops,
             "flops_source": "ncu counts on the current sources (profiles/traffic.json)"}
 
 E2E_REPEATS = 3
@@ -927,7 +932,7 @@ def main():
         alu = fp64_alu(tkey, cells, col_ms, fp64_peak) or {}
         roofline = {"bound": "alu", "kernel": "k_collide (fused collide-and-stream, FP64)",
                     "achieved": alu.get("achieved_tflops"), "peak": fp64_peak, "unit": "TFLOP/s",
-                    "frac": alu.get("frac"),
+                    "frac": alu.get("frac"), "pipe_frac": alu.get("pipe_frac"),
                     "peak_source": "measured in this run: FP64 FMA chains at full occupancy "
                                    "(lbnr_fp64_fma_rate)",
                     "flops_per_cell": alu.get("flops_per_cell"),

@@ -230,7 +230,7 @@ __device__ __forceinline__ void bm_sources_plain(const T alpha, const T g[6], co
 // its scheduler for 64 cycles, whatever the active lanes): with 200 cells of
 // D1Q3 a step takes 28 us instead of 42, 64^3 with the monitor 50.3 ms instead
 // of 55.4 for 40 steps. 16-bit storage waits on the latency of its instructions
-// (32 to 38 % of the issue slots used), so fewer in a row help there too: 256^3
+// (41 % of the issue slots used), so fewer in a row help there too: 256^3
 // D3Q19 FP16, 100 steps 653 instead of 697 ms, host copies included.
 template <class T, int dim>
 __device__ __forceinline__ void bm_sources(const T alpha, const T g[6], const T K[6],
