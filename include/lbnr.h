@@ -244,7 +244,7 @@ int lbnr_has_shift(const lbnr_ctx* ctx);
  * autotuner. Names: "P1-hold" / "P1-reread" (distributions held in registers
  * between the moment and update passes, or read again), with a suffix
  * "-<t>x<b>" for blocks of t threads sized for b blocks per SM (no suffix: 128
- * x 3, FP64 64 x 6); "tma-p1-nc<c>-k<k>-t32" (persistent, fed by bulk copies of
+ * x 3, under LAG 128 x 2 for 4-byte storage on D3Q19; FP64 64 x 6); "tma-p1-nc<c>-k<k>-t32" (persistent, fed by bulk copies of
  * whole 32-cell tiles, c consumer warps with k stages each); "lanes<n>" (FP64:
  * n lanes share a cell; in place form 0 runs instead). The others run one
  * thread per cell. The bulk-copy-fed forms read each tile's own cells only; at
